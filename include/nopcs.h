@@ -325,8 +325,9 @@ nopcs_status nopcs_plane_fields(nopcs_ctx *ctx, int box, int axis, int index, in
  * the sub-domain length per axis (the autotuner's pick where the descriptor
  * asked for -1), the form of the FP32 derivative per axis (NOPCS_FORM_THOMAS,
  * NOPCS_FORM_GEMM_3XTF32, NOPCS_FORM_GEMM_BF16X3 or NOPCS_FORM_BANDED) and the
- * flux sweeps' tile width per axis (grid lines per CUDA block; 0 = the
- * precision's default, untuned for small boxes).
+ * flux sweeps' tile width per axis (grid lines per CUDA block in the FP64
+ * form; 0 = the default, untuned for small boxes, and always in the mixed form,
+ * whose flux sweeps are not tiled by lines and sub-domains).
  */
 nopcs_status nopcs_box_info(nopcs_ctx *ctx, int box, int *sub_n, int *deriv_form, int *tile_lines);
 

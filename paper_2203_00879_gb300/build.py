@@ -66,10 +66,11 @@ if __name__ == "__main__":
 
 
 _LINE = ["line_kernels.cu", "line_body.cuh", "line_solve.cuh"]
+_SWEEP = ["sweep32.cuh", "sweep32_kernels.cu"]  # FP32 (mixed form)
 KERNEL_FILES = {
     "prep": ["rk_kernels.cu", "fp_bits.cuh"], "wall_bc": ["rk_kernels.cu", "wall_body.cuh", "fp_bits.cuh"],
     "diagnostics": ["rk_kernels.cu", "fp_bits.cuh"],
-    "sweep_x": _LINE + ["xline_kernels.cu"], "sweep_y": _LINE, "sweep_z": _LINE,
+    "sweep_x": _SWEEP, "sweep_y": _SWEEP, "sweep_z": _SWEEP,
     "filter": _LINE + ["rk_kernels.cu"], "visc_rk_update": ["visc_kernel.cu", "visc_body.cuh", "fp_bits.cuh"],
 }
 

@@ -63,7 +63,7 @@ struct BoxRes {
     LineOpBuf d2op64[3], d2op32[3];  // compact second derivative (nopcs_derivative order 3)
     GemmOpBuf gop[3];  // dense blocks of the FP32 derivative (tensor-core form)
     int sub_n[3] = {0, 0, 0};     // sub-domain length in use per axis (tuned if asked)
-    int lines[3] = {0, 0, 0};     // flux-sweep lines per block per axis (0: default)
+    int lines[3] = {0, 0, 0};     // FP64 flux-sweep lines per block per axis (0: default)
     bool deriv_gemm[3] = {false, false, false};  // FP32 derivative on the tensor cores
     bool gemm_bf16[3] = {false, false, false};   // ... in the BF16x3 split (else 3xTF32)
     bool deriv_band[3] = {false, false, false};  // FP32 derivative in the banded explicit form
@@ -294,14 +294,15 @@ cudaError_t refresh_mixed(BoxRes &b, cudaStream_t st)
 }
 
 // ---- autotuner ---------------------------------------------------------------
-// Per axis, the flux sweep's tile width (16 or 32 lines per block) and, where
-// the descriptor asks with sub_n = -1, the sub-domain length (32, 64 or 128)
-// are chosen by timing the sweep the RK path uses (the context precision) on
-// this GPU; under NOPCS_FORM_AUTO each axis's FP32 derivative takes the Thomas
-// or the tensor-core form, whichever measured faster.  Times come from CUDA
-// events on the context stream (one warm-up, three timed launches); choices
-// are cached per box shape for the process.  Boxes below 2^20 points keep the
-// defaults unless a sub-domain length is requested.
+// Per axis: in the FP64 form, the flux sweep's tile width (16 or 32 lines per
+// block); where the descriptor asks with sub_n = -1, the sub-domain length
+// (32, 64 or 128), by timing the flux sweep (FP64 form, together with the tile
+// width) or the FP32 derivative (mixed form, whose flux sweeps do not depend
+// on the partition).  Under NOPCS_FORM_AUTO each axis's FP32 derivative takes
+// the Thomas, the banded or a tensor-core form, whichever measured faster.
+// Times come from CUDA events on the context stream (one warm-up, three timed
+// launches); choices are cached per box shape for the process.  Boxes below
+// 2^20 points keep the defaults unless a sub-domain length is requested.
 std::mutex g_tune_mu;
 std::map<std::string, int> g_tune_cache;
 
@@ -329,11 +330,14 @@ nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
     const BoxDev &x = b.dev;
     char key0[96];
     snprintf(key0, sizeof(key0), "%d,%d,%d,%d", x.n[0], x.n[1], x.n[2], b.mixed ? 1 : 0);
-    // primitives of the current state feed the timed sweeps
+    // scratch FP32 fields inside the right-hand-side buffer (>= 2 np floats)
+    float *fin = (float *)b.R, *fout = fin + x.np;
+    // primitives of the current state feed the timed FP64 sweeps
     if (!b.mixed) CK(launch_prep<double>(x, b.Qn(), (double *)b.W, nullptr, st), "autotune");
+    if (b.mixed) CK(cudaMemsetAsync(fin, 0, (size_t)x.np * sizeof(float), st), "autotune");
     for (int a = 0; a < 3; ++a) {
         const bool tune_sub = b.d.sub_n[a] == -1;
-        if (!tune_sub && x.np < (1LL << 20)) continue;
+        if (!tune_sub && (b.mixed || x.np < (1LL << 20))) continue;
         const std::string key = std::string(key0) + ",s" + std::to_string(a) + "," + std::to_string(b.d.sub_n[a]);
         int best = -1;  // sub_n * 1000 + lines per block
         {
@@ -356,8 +360,9 @@ nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
                     if (s2 != NOPCS_OK) return s2;
                 }
                 for (int ln : {16, 32}) {
+                    if (b.mixed && ln == 16) continue;
                     cudaError_t e;
-                    float ms = b.mixed ? time_launches(st, [&] { return launch_line_flux<float>(b.dop32[a].dev, a, x, b.Wm(0), b.Rm(), 1, st, ln); }, e)
+                    float ms = b.mixed ? time_launches(st, [&] { return launch_line_field<float>(b.dop32[a].dev, a, x.n, fin, fout, 1.0, st); }, e)
                                        : time_launches(st, [&] { return launch_line_flux<double>(b.dop64[a].dev, a, x, (double *)b.W, (double *)b.R, 1, st, ln); }, e);
                     if (e != cudaSuccess) return cuda_fail(ctx, e, "autotune");
                     if (ms < tbest) {
@@ -369,7 +374,7 @@ nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
             std::lock_guard<std::mutex> lk(g_tune_mu);
             g_tune_cache[key] = best;
         }
-        b.lines[a] = best % 1000;
+        if (!b.mixed) b.lines[a] = best % 1000;
         if (!tune_sub) continue;
         best /= 1000;
         b.sub_n[a] = best;
@@ -377,8 +382,6 @@ nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
         if (s2 != NOPCS_OK) return s2;
     }
     if (ctx->form == NOPCS_FORM_AUTO) {
-        // scratch FP32 fields inside the right-hand-side buffer (>= 2 np floats)
-        float *fin = (float *)b.R, *fout = fin + x.np;
         CK(cudaMemsetAsync(fin, 0, 2 * (size_t)x.np * sizeof(float), st), "autotune");
         for (int a = 0; a < 3; ++a) {
             b.deriv_gemm[a] = false;
@@ -1269,10 +1272,7 @@ nopcs_status nopcs_set_launch(nopcs_ctx *ctx, int mode, double wait_limit_s)
                             "the persistent launch runs mixed-precision boxes with the explicit viscous terms");
             BatchBoxIn x;
             x.bx = b.dev;
-            for (int a = 0; a < 3; ++a) {
-                x.op[a] = b.dop32[a].dev;
-                x.lines[a] = b.lines[a];
-            }
+            for (int a = 0; a < 3; ++a) x.op[a] = b.dop32[a].dev;
             x.W[0] = b.Wm(0);
             x.W[1] = b.Wm(1);
             x.R = b.Rm();

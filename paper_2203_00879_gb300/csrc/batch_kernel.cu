@@ -8,7 +8,7 @@
 // phase, a run of blocks), each box's phases in order; every block of the
 // persistent grid takes the next item from an atomic counter, waits until the
 // box's previous phase has completed all its items, runs the item's blocks
-// with the same device code as the stand-alone kernels (line_body.cuh,
+// with the same device code as the stand-alone kernels (sweep32.cuh,
 // visc_body.cuh, wall_body.cuh), and counts the item done.  Boxes advance
 // independently, so small boxes fill the GPU side by side without a launch
 // per kernel and box.
@@ -20,10 +20,11 @@
 // every later wait returns at once, and the kernel ends.  The completion
 // counters use release / acquire at GPU scope; the data of a finished phase is
 // read by plain (coherent) loads after the acquiring thread's barrier.
+#include <algorithm>
 #include <string>
 #include <vector>
 
-#include "line_body.cuh"
+#include "sweep32.cuh"
 #include "visc_body.cuh"
 #include "wall_body.cuh"
 
@@ -32,6 +33,12 @@ namespace nopcs {
 namespace {
 
 constexpr int BT = 256;             // threads per block (the viscous tile's)
+// Lines per tile of the y and z sweeps (half as many with a ring of 8 groups)
+// and rows of theirs in flight, at two blocks per SM: a step of the 64-box
+// workload takes 39.4 ms, of one 256^3 box 9.1 ms; with 160 lines 39.4 and 9.8,
+// with 160 lines and 8 rows 42.2 and 10.7, at three blocks per SM (80 registers
+// a thread, the sweeps spill) with 96 lines and 2 rows 46.5 and 11.6.
+constexpr int BMARCH = 128, BU = 4;
 // wall nodes per tile of the face and edge phases: four passes of a block,
 // so that a box's wall phases spread over many blocks instead of holding the
 // box's next phase behind a few long items
@@ -39,17 +46,14 @@ constexpr int WALL_CHUNK = 4 * BT;
 enum { PH_SX = 0, PH_SY, PH_SZ, PH_VISC, PH_FACE, PH_EDGE, PH_CORNER, NPH };
 
 struct BStage {
-    LineArgs<float> la[3];
+    Sweep32Args sw[3];
     VArgs<float> va;
     double *Q;  // wall conditions: the FP64 state (stage 4) or null (stage state Ww)
     float *Dn, *Wf, *Ww;
 };
 
 struct BBox {
-    LineOpDev op[3];
     BoxDev bx;
-    int nt[3];       // working threads of each sweep (those of its stand-alone launch)
-    int xline;       // the x sweep is the whole-line kernel
     int ntile[NPH];  // blocks of the stand-alone launch per phase
     int chunk[NPH];  // blocks per item
     int nitem[NPH];  // items per phase
@@ -112,23 +116,27 @@ __device__ bool wait_at_least(const BParams &p, const int *ctr, int need)
 // The phase bodies are separate (not inlined) functions, so that each gets the
 // kernel's whole register budget instead of all of them sharing one
 // allocation inside the item loop.
-__device__ __noinline__ void run_sweep_x(const LineOpDev &op, const LineArgs<float> &la, int v, unsigned char *sm,
-                                         int nt, int xline)
+__device__ __noinline__ void run_sweep_x(const Sweep32Args &a, int v, float *sm)
 {
-    if (xline)
-        xline_body<float, MODE_FLUX>(op, la, v);
-    else
-        line_body<float, MODE_FLUX, 0>(op, la, v, nt);
+    const int w = (int)(threadIdx.x >> 5);
+    scan_any<MODE_FLUX>(a, v * (BT / 32) + w, sm + w * SweepMode<MODE_FLUX>::NF * SC_FS);
 }
-__device__ __noinline__ void run_sweep_y(const LineOpDev &op, const LineArgs<float> &la, int v, unsigned char *sm,
-                                         int nt)
+template <int AXIS>
+__device__ __noinline__ void run_march(const Sweep32Args &a, int v, float *sm)
 {
-    line_body<float, MODE_FLUX, 1>(op, la, v, nt);
-}
-__device__ __noinline__ void run_sweep_z(const LineOpDev &op, const LineArgs<float> &la, int v, unsigned char *sm,
-                                         int nt)
-{
-    line_body<float, MODE_FLUX, 2>(op, la, v, nt);
+    if (threadIdx.x >= BMARCH) return;
+    if (a.ring == 8) {
+        if (threadIdx.x >= BMARCH / 2) return;
+        if (a.ga == AXIS)
+            march_body<MODE_FLUX, AXIS, true, 8, BMARCH / 2, BU, false>(a, (unsigned)v, (int)threadIdx.x, sm);
+        else
+            march_body<MODE_FLUX, AXIS, false, 8, BMARCH / 2, BU, false>(a, (unsigned)v, (int)threadIdx.x, sm);
+    } else {
+        if (a.ga == AXIS)
+            march_body<MODE_FLUX, AXIS, true, 4, BMARCH, BU, false>(a, (unsigned)v, (int)threadIdx.x, sm);
+        else
+            march_body<MODE_FLUX, AXIS, false, 4, BMARCH, BU, false>(a, (unsigned)v, (int)threadIdx.x, sm);
+    }
 }
 // the viscous stage kernel in the same specialisation as the stand-alone
 // launch (per stage, gravity along z) or the generic one
@@ -150,17 +158,16 @@ __device__ __forceinline__ void run_visc_any(const VArgs<float> &va, int bx, int
     run_visc<RunSpec>(va, bx, by, bz, sm);
 }
 
-__global__ void __launch_bounds__(BT, 3) batch_step_kernel(const BParams p)
+__global__ void __launch_bounds__(BT, 2) batch_step_kernel(const BParams p)
 {
     extern __shared__ __align__(32) unsigned char smraw[];
     __shared__ int s_item, s_go;
     // the item's arguments, copied from the device box table: the phase code
     // then reads its pointers and constants from shared memory instead of
     // through global loads ahead of every data access
-    constexpr int ARGW = (int)((sizeof(VArgs<float>) > sizeof(LineOpDev) + sizeof(LineArgs<float>)
-                                    ? sizeof(VArgs<float>)
-                                    : sizeof(LineOpDev) + sizeof(LineArgs<float>)) /
-                               8);
+    constexpr int ARGW =
+        (int)((sizeof(VArgs<float>) > sizeof(Sweep32Args) ? sizeof(VArgs<float>) : sizeof(Sweep32Args)) / 8);
+    static_assert(sizeof(VArgs<float>) % 8 == 0 && sizeof(Sweep32Args) % 8 == 0, "copied in 8-byte words");
     __shared__ unsigned long long s_args[ARGW];
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(p.next, 1);
@@ -193,8 +200,7 @@ __global__ void __launch_bounds__(BT, 3) batch_step_kernel(const BParams p)
         __syncthreads();
         if (s_go) {
             const BStage &S = B.st[it.stage];
-            LineOpDev *sop = reinterpret_cast<LineOpDev *>(s_args);
-            LineArgs<float> *sla = reinterpret_cast<LineArgs<float> *>(s_args + sizeof(LineOpDev) / 8);
+            Sweep32Args *ssw = reinterpret_cast<Sweep32Args *>(s_args);
             VArgs<float> *sva = reinterpret_cast<VArgs<float> *>(s_args);
             {
                 auto copy = [&](void *dst, const void *src, int bytes) {
@@ -203,8 +209,7 @@ __global__ void __launch_bounds__(BT, 3) batch_step_kernel(const BParams p)
                     for (int k = threadIdx.x; k < bytes / 8; k += BT) b[k] = a[k];
                 };
                 if (it.phase <= PH_SZ) {
-                    copy(sop, &B.op[it.phase], (int)sizeof(LineOpDev));
-                    copy(sla, &S.la[it.phase], (int)sizeof(LineArgs<float>));
+                    copy(ssw, &S.sw[it.phase], (int)sizeof(Sweep32Args));
                 } else if (it.phase == PH_VISC) {
                     copy(sva, &S.va, (int)sizeof(VArgs<float>));
                 }
@@ -213,9 +218,9 @@ __global__ void __launch_bounds__(BT, 3) batch_step_kernel(const BParams p)
             const int last = min(it.first + B.chunk[it.phase], B.ntile[it.phase]);
             for (int v = it.first; v < last; ++v) {
                 switch (it.phase) {
-                case PH_SX: run_sweep_x(*sop, *sla, v, smraw, B.nt[0], B.xline); break;
-                case PH_SY: run_sweep_y(*sop, *sla, v, smraw, B.nt[1]); break;
-                case PH_SZ: run_sweep_z(*sop, *sla, v, smraw, B.nt[2]); break;
+                case PH_SX: run_sweep_x(*ssw, v, reinterpret_cast<float *>(smraw)); break;
+                case PH_SY: run_march<1>(*ssw, v, reinterpret_cast<float *>(smraw)); break;
+                case PH_SZ: run_march<2>(*ssw, v, reinterpret_cast<float *>(smraw)); break;
                 case PH_VISC: run_visc_any(*sva, v % B.gx, (v / B.gx) % B.gy, v / (B.gx * B.gy), smraw); break;
                 case PH_FACE: {
                     const long long tot = face_count(B.bx);
@@ -273,44 +278,27 @@ cudaError_t batch_plan_build(const std::vector<BatchBoxIn> &in, BatchPlan **out,
     const int nb = (int)in.size();
     std::vector<BBox> boxes(nb);
     std::vector<BItem> items;
-    size_t smem = ring_bytes<float>();
+    constexpr int NF = SweepMode<MODE_FLUX>::NF;
+    const size_t smem = std::max({ring_bytes<float>(), scan_smem(NF, BT / 32), march_smem(NF, 4, BMARCH)});
     for (int b = 0; b < nb; ++b) {
         const BatchBoxIn &I = in[b];
         BBox &B = boxes[b];
         B.bx = I.bx;
-        for (int a = 0; a < 3; ++a) B.op[a] = I.op[a];
-        const long long np = I.bx.np;
         for (int s = 1; s <= 4; ++s) {
             BStage &S = B.st[s - 1];
             const float *Win = I.W[(s - 1) & 1];
             float *Wout = I.W[s & 1];
             for (int a = 0; a < 3; ++a) {
-                LineArgs<float> &la = S.la[a];
-                la = LineArgs<float>{};
-                for (int d = 0; d < 3; ++d) la.n[d] = I.bx.n[d];
-                for (int k = 0; k < 6; ++k) la.in[k] = Win + (size_t)k * np;
-                for (int k = 0; k < 5; ++k) la.out[k] = I.R + (size_t)k * np;
-                la.scale = (float)I.bx.inv_h[a];
-                la.first = a == 0;
-                la.ga = I.bx.ga;
-                la.b0 = I.bx.rho_b32;
-                la.b1 = I.bx.H_b32;
-                // the stand-alone launch's geometry (same tile width and
-                // working threads, so the same arithmetic and rounding)
-                LineGrid g;
-                const int pref = I.lines[a] > 0 ? I.lines[a] : 32;
-                bool ok = a == 0 ? line_grid<float, MODE_FLUX, 0>(I.op[a], la, pref, 0, XLINE_MAX_LINES, g)
-                                 : (a == 1 ? line_grid<float, MODE_FLUX, 1>(I.op[a], la, pref, 0, XLINE_MAX_LINES, g)
-                                           : line_grid<float, MODE_FLUX, 2>(I.op[a], la, pref, 0, XLINE_MAX_LINES, g));
-                const int cols = g.xline ? I.op[0].nsub * 5 * la.lines : 0;
-                if (!ok || g.nblk > 0x7fffffff || (g.xline ? cols > BT : g.threads > BT)) {
+                // the stand-alone launch's pieces (the same arithmetic)
+                Sweep32Args &w = S.sw[a];
+                w = Sweep32Args{};
+                if (!flux32_args(I.op[a], a, I.bx, Win, I.R, w)) {
                     msg = "a flux sweep of a box does not fit the batched kernel's blocks";
                     return cudaErrorInvalidConfiguration;
                 }
-                if (g.smem > smem) smem = g.smem;
-                B.ntile[PH_SX + a] = (int)g.nblk;
-                B.nt[a] = g.threads;
-                if (a == 0) B.xline = g.xline ? 1 : 0;
+                const long long per = SC_USE * (BT / 32), bm = w.ring == 8 ? BMARCH / 2 : BMARCH;
+                B.ntile[PH_SX + a] = (int)(a == 0 ? (w.tot + per - 1) / per
+                                                  : (w.cols + bm - 1) / bm * w.nseg);
             }
             StageRegs<float> r;
             r.Qn = I.Qn;

@@ -1,9 +1,7 @@
 // Device bodies of the NOHAP line sweeps (arXiv 2203.00879, Sec. 3): the
 // sub-domain sweep (line_body) and the whole-line x sweep (xline_body), each
-// for one block given as a block index of its launch grid, so that the
-// stand-alone kernels (line_kernels.cu) and the batched persistent kernel
-// (batch_kernel.cu) run the same code.  The header comment of line_kernels.cu
-// describes the algorithm.
+// for one block given as a block index of its launch grid.  The header comment
+// of line_kernels.cu describes the algorithm.
 #pragma once
 
 #include "line_solve.cuh"

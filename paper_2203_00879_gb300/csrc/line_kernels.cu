@@ -20,10 +20,11 @@
 // tile and takes the end values from it.)
 //
 // Modes: FIELD / FIELD2 one field; FLUX the five inviscid fluxes along the
-// axis from the stage primitives, into R; FILTER five state fields; VGRAD and
+// axis from the stage primitives, into R (FP64; FP32 in sweep32.cuh); FILTER five state fields; VGRAD and
 // VDIV the compact viscous terms -- the derivatives of u, v, w, T, and those
 // of the four viscous-flux components along the axis, added into R[1..4].
 #include "line_body.cuh"
+#include "sweep32.cuh"
 
 namespace nopcs {
 
@@ -78,7 +79,6 @@ cudaError_t init_line_kernels()
     cudaError_t r[] = {
         allow_smem<float, MODE_FIELD, 0>(),  allow_smem<float, MODE_FIELD, 1>(),  allow_smem<float, MODE_FIELD, 2>(),
         allow_smem<double, MODE_FIELD, 0>(), allow_smem<double, MODE_FIELD, 1>(), allow_smem<double, MODE_FIELD, 2>(),
-        allow_smem<float, MODE_FLUX, 0>(),   allow_smem<float, MODE_FLUX, 1>(),   allow_smem<float, MODE_FLUX, 2>(),
         allow_smem<double, MODE_FLUX, 0>(),  allow_smem<double, MODE_FLUX, 1>(),  allow_smem<double, MODE_FLUX, 2>(),
         allow_smem<double, MODE_FILTER, 0>(), allow_smem<double, MODE_FILTER, 1>(),
         allow_smem<double, MODE_FILTER, 2>(),  allow_smem<float, MODE_FILTER, 0>(),
@@ -113,21 +113,24 @@ template <typename T>
 cudaError_t launch_line_flux(const LineOpDev &op, int axis, const BoxDev &bx, const T *W, T *R,
                              int first, cudaStream_t st, int lines)
 {
-    LineArgs<T> a{};
-    for (int d = 0; d < 3; ++d) a.n[d] = bx.n[d];
-    for (int k = 0; k < 6; ++k) a.in[k] = W + (size_t)k * bx.np;
-    for (int k = 0; k < 5; ++k) a.out[k] = R + (size_t)k * bx.np;
-    a.scale = (T)bx.inv_h[axis];
-    a.first = first;
-    a.ga = bx.ga;
-    if (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 4) {
+        // FP32: recurrences without end rows (sweep32.cuh); the x sweep
+        // stores and the others add, as `first` says
+        Sweep32Args s{};
+        if ((first != 0) != (axis == 0) || !flux32_args(op, axis, bx, W, R, s)) return cudaErrorInvalidValue;
+        return launch_sweep32<MODE_FLUX>(axis, s, st);
+    } else {
+        LineArgs<T> a{};
+        for (int d = 0; d < 3; ++d) a.n[d] = bx.n[d];
+        for (int k = 0; k < 6; ++k) a.in[k] = W + (size_t)k * bx.np;
+        for (int k = 0; k < 5; ++k) a.out[k] = R + (size_t)k * bx.np;
+        a.scale = (T)bx.inv_h[axis];
+        a.first = first;
+        a.ga = bx.ga;
         a.b0 = (const T *)bx.rho_b64;
         a.b1 = (const T *)bx.H_b64;
-    } else {
-        a.b0 = (const T *)bx.rho_b32;
-        a.b1 = (const T *)bx.H_b32;
+        return launch_any<T, MODE_FLUX>(op, axis, a, lines > 0 ? lines : 16, st);
     }
-    return launch_any<T, MODE_FLUX>(op, axis, a, lines > 0 ? lines : (sizeof(T) == 4 ? 32 : 16), st);
 }
 
 cudaError_t launch_line_filter(const LineOpDev &op, int axis, const BoxDev &bx, int base_subtract,

@@ -203,7 +203,8 @@ template <typename T>
 cudaError_t launch_line_field2(const LineOpDev &op, int axis, const int n[3], const T *f, T *out, double scale,
                                cudaStream_t st);
 // FLUX: R (= or -=) L(flux_axis(W)) / h.  first != 0 stores, else subtracts.
-// lines: lines per block (tile width; 0 = default for the precision).
+// FP64: lines per block (tile width; 0 = default).  FP32 (sweep32.cuh): the x
+// sweep stores, the others subtract.
 template <typename T>
 cudaError_t launch_line_flux(const LineOpDev &op, int axis, const BoxDev &bx, const T *W, T *R,
                              int first, cudaStream_t st, int lines = 0);
@@ -285,11 +286,10 @@ void dev_free(void *p);
 
 // ---- one persistent launch per RK step (batch_kernel.cu) -------------------------
 // One mixed-form box as the batched kernel sees it: its constants, FP32
-// derivative operators, flux-sweep tile widths (0: default) and registers.
+// derivative operators and registers.
 struct BatchBoxIn {
     BoxDev bx;
     LineOpDev op[3];
-    int lines[3];
     float *W[2], *R, *K, *Dn;
     double *Qn;
 };

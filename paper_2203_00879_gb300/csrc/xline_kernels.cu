@@ -28,11 +28,8 @@ cudaError_t init_xline_flux()
     return cudaFuncSetAttribute(xline_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XLINE_SMEM);
 }
 
-template cudaError_t launch_xline_flux<float>(const LineOpDev &, const LineArgs<float> &, long long, int, size_t,
-                                              cudaStream_t);
 template cudaError_t launch_xline_flux<double>(const LineOpDev &, const LineArgs<double> &, long long, int, size_t,
                                                cudaStream_t);
-template cudaError_t init_xline_flux<float>();
 template cudaError_t init_xline_flux<double>();
 
 }  // namespace nopcs
