@@ -138,24 +138,28 @@ __device__ __noinline__ void run_march(const Sweep32Args &a, int v, float *sm)
             march_body<MODE_FLUX, AXIS, false, 4, BMARCH, BU, false>(a, (unsigned)v, (int)threadIdx.x, sm);
     }
 }
-// the viscous stage kernel in the same specialisation as the stand-alone
-// launch (per stage, gravity along z) or the generic one
+// the viscous stage kernel in the specialisations of the stand-alone launch
 template <class S>
 __device__ __noinline__ void run_visc(const VArgs<float> &va, int bx, int by, int bz, unsigned char *sm)
 {
     visc_rk_block<float, S>(va, bx, by, bz, sm);
 }
+template <int GA>
+__device__ __forceinline__ void run_visc_ga(const VArgs<float> &va, int bx, int by, int bz, unsigned char *sm)
+{
+    switch (va.stage) {
+    case 1: run_visc<Spec<1, GA>>(va, bx, by, bz, sm); return;
+    case 2: run_visc<Spec<2, GA>>(va, bx, by, bz, sm); return;
+    case 3: run_visc<Spec<3, GA>>(va, bx, by, bz, sm); return;
+    default: run_visc<Spec<4, GA>>(va, bx, by, bz, sm);
+    }
+}
 __device__ __forceinline__ void run_visc_any(const VArgs<float> &va, int bx, int by, int bz, unsigned char *sm)
 {
-    if (va.ga == 2) {
-        switch (va.stage) {
-        case 1: run_visc<Spec<1, 2>>(va, bx, by, bz, sm); return;
-        case 2: run_visc<Spec<2, 2>>(va, bx, by, bz, sm); return;
-        case 3: run_visc<Spec<3, 2>>(va, bx, by, bz, sm); return;
-        case 4: run_visc<Spec<4, 2>>(va, bx, by, bz, sm); return;
-        }
-    }
-    run_visc<RunSpec>(va, bx, by, bz, sm);
+    if (va.ga == 2)
+        run_visc_ga<2>(va, bx, by, bz, sm);
+    else
+        run_visc_ga<-1>(va, bx, by, bz, sm);
 }
 
 __global__ void __launch_bounds__(BT, 2) batch_step_kernel(const BParams p)
@@ -279,7 +283,7 @@ cudaError_t batch_plan_build(const std::vector<BatchBoxIn> &in, BatchPlan **out,
     std::vector<BBox> boxes(nb);
     std::vector<BItem> items;
     constexpr int NF = SweepMode<MODE_FLUX>::NF;
-    const size_t smem = std::max({ring_bytes<float>(), scan_smem(NF, BT / 32), march_smem(NF, 4, BMARCH)});
+    const size_t smem = std::max({visc_smem<float>(), scan_smem(NF, BT / 32), march_smem(NF, 4, BMARCH)});
     for (int b = 0; b < nb; ++b) {
         const BatchBoxIn &I = in[b];
         BBox &B = boxes[b];
@@ -306,15 +310,10 @@ cudaError_t batch_plan_build(const std::vector<BatchBoxIn> &in, BatchPlan **out,
             r.Dn = I.Dn;
             r.Wn = Wout;
             S.va = make_vargs<float>(I.bx, Win, I.R, s, r);
-            B.gx = (I.bx.n[0] + TX - 1) / TX;
-            B.gy = (I.bx.n[1] + TY - 1) / TY;
-            // z chunk of the stand-alone launch (8 to 32 planes per block)
-            const long long want = 152LL * 8;
-            const int nzc = (int)((want + (long long)B.gx * B.gy - 1) / ((long long)B.gx * B.gy));
-            int zc = (I.bx.n[2] + nzc - 1) / nzc;
-            zc = zc < 8 ? 8 : (zc > 32 ? 32 : zc);
-            S.va.zc = zc;
-            B.ntile[PH_VISC] = B.gx * B.gy * ((I.bx.n[2] + zc - 1) / zc);
+            const dim3 vg = visc_grid<float>(I.bx, S.va.zc);
+            B.gx = (int)vg.x;
+            B.gy = (int)vg.y;
+            B.ntile[PH_VISC] = (int)(vg.x * vg.y * vg.z);
             if (s < 4) {
                 S.Q = nullptr;
                 S.Dn = nullptr;

@@ -6,34 +6,46 @@
 // divergence of nodal viscous fluxes, and each nodal flux needs second-order
 // explicit gradients of u, v, w, T at its node: a +-2 stencil (+-3 next to a
 // wall, where both operators are one-sided).  A block owns a TX x TY column
-// tile and marches along z, keeping the primitives (u, v, w, T) of the five
-// planes o-2 .. o+2 around the output plane o, with a two-node x/y halo, in a
-// shared-memory ring; every primitive is loaded from global memory once per
-// block and plane.  For each plane the block then
-//   1. evaluates every nodal viscous flux once: E_v on the plane's tile plus
-//      a one-node x halo, F_v on the tile plus a one-node y halo, and G_v on
-//      the tile of the planes the z divergence needs, kept in a ring of three
-//      planes so each G_v plane is computed once and used twice;
-//   2. takes the divergence at its tile nodes, adds the gravity source to the
-//      convective right-hand side accumulated by the sweeps, holds momentum at
-//      zero on wall nodes (no-slip) and applies the RK4 stage.
-// The primitive loads of the next plane are issued during step 2.
+// tile, a thread per node of a plane, and marches along z.  In step j
+//   1. E_v, F_v and G_v of plane j are evaluated from one stencil in the ring of
+//      primitives (u, v, w, T; four planes with a two-node x/y halo in shared
+//      memory, each primitive loaded once per block and plane), E_v also on the
+//      x halo and F_v on the y halo; G_v stays in the thread's registers;
+//   2. plane j - 1, whose z divergence is now complete, gets the gravity source
+//      on top of the convective right-hand side accumulated by the sweeps,
+//      zero momentum on wall nodes (no-slip) and the RK4 stage;
+//   3. plane j + 2 goes into the ring, and after the step's only barrier
+//   4. the x and y divergence of plane j is taken from E_v and F_v in shared
+//      memory (two planes, so that the next step can write while others read).
+// The loads of steps 2 and 3 are issued before step 1, and L2 is asked for
+// those of the next step.
 //
 // Tiles never start past n - TX, so every tile is at least min(n, TX) wide and
 // the one-sided wall stencils stay inside it; a tile that had to be shifted
 // back writes only the columns it owns.
+//
+// Bound by issue slots and latency (stage 2 at 256^3: 56% of the issue slots,
+// 568 instructions a node, 57% of the HBM cycles; 24 warps an SM, held by 80
+// registers).  Mean over the stages at 1024 x 512 x 512: 6.98 ms (138 B a
+// point, 0.78 of the measured copy bandwidth) against 8.04 with a five-plane
+// ring, G_v in shared memory and two barriers per plane; at 256^3 0.526
+// against 0.594, at 48^3 17 us against 31.  Measured slower: two rows a thread
+// in 32 x 16 tiles (128 registers, 16 warps: 431 instructions a node, but 7.58
+// ms); four blocks per SM (spills, 12.6); the next plane's inputs copied to
+// shared memory with cp.async (9.8: 4-byte copies saturate the memory pipe);
+// plane base + 32-bit offset addresses (more instructions).  Stage 4 at 256^3:
+// 0.736 ms against 0.827; its binary32/binary64 conversions had been issued to
+// the FP64 pipe for every value (49% busy, now 26%).
 #include "visc_body.cuh"
 
 namespace nopcs {
 
 namespace {
 
-// FP32: three blocks (24 warps) per SM, with up to 85 registers per thread;
-// a 64-register cap for four blocks was 1.4% slower once the L2 prefetches
-// had taken the load latency off the update.  S fixes the stage and the
-// gravity axis at compile time (Spec) or leaves them to the arguments.
+// S fixes the stage and the gravity axis at compile time (Spec) or leaves
+// them to the arguments.
 template <typename T, class S>
-__global__ void __launch_bounds__(TX *TY, (sizeof(T) == 4 ? 768 : 512) / (TX * TY)) visc_rk_kernel(const VArgs<T> a)
+__global__ void __launch_bounds__(VT, visc_occupancy<T>()) visc_rk_kernel(const __grid_constant__ VArgs<T> a)
 {
     extern __shared__ __align__(32) unsigned char smraw[];
     visc_rk_block<T, S>(a, blockIdx.x, blockIdx.y, blockIdx.z, smraw);
@@ -91,6 +103,7 @@ __global__ void __launch_bounds__(256) source_rk_kernel(const VArgs<T> a)
         const int p = (int)q;  // boxes hold < 2^31 points
         T r[5];
         float kd[5], dn[5];
+        double qn[5];
 #pragma unroll
         for (int k = 0; k < 5; ++k) r[k] = a.R[k][p];
         if constexpr (sizeof(T) == 4) {
@@ -102,11 +115,15 @@ __global__ void __launch_bounds__(256) source_rk_kernel(const VArgs<T> a)
 #pragma unroll
                 for (int k = 0; k < 5; ++k) dn[k] = a.Dn[k][p];
             }
+            if (a.stage == 4) {
+#pragma unroll
+                for (int k = 0; k < 5; ++k) qn[k] = a.Qn[k][p];
+            }
         }
         const int x = p % nx, y = (p / nx) % ny, z = p / (nx * ny);
         const int kg = a.ga == 0 ? x : (a.ga == 1 ? y : z);
         const bool wall = x == 0 || x == nx - 1 || y == 0 || y == ny - 1 || z == 0 || z == nz - 1;
-        source_and_stage(a, p, kg, wall, a.W[0][p], a.W[1 + a.ga][p], r, kd, dn);
+        source_and_stage(a, p, kg, wall, a.W[0][p], a.W[1 + a.ga][p], r, kd, dn, qn);
     }
 }
 
@@ -118,23 +135,23 @@ unsigned pointwise_blocks(long long np)
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-// The stage kernel for (stage, gravity axis): FP32 with gravity along z, the
-// benchmark's case, specialised per stage; everything else generic.
+// The stage kernel for (stage, gravity axis): the FP32 ones are specialised
+// per stage, and for gravity along z; the FP64 one is generic.
 template <typename T>
 const void *visc_kernel_for(int stage, int ga)
 {
     if constexpr (sizeof(T) == 4) {
-        if (ga == 2) {
-            switch (stage) {
-            case 0: return (const void *)visc_rk_kernel<float, Spec<0, 2>>;
-            case 1: return (const void *)visc_rk_kernel<float, Spec<1, 2>>;
-            case 2: return (const void *)visc_rk_kernel<float, Spec<2, 2>>;
-            case 3: return (const void *)visc_rk_kernel<float, Spec<3, 2>>;
-            case 4: return (const void *)visc_rk_kernel<float, Spec<4, 2>>;
-            }
+        const bool z = ga == 2;
+        switch (stage) {
+        case 0: return z ? (const void *)visc_rk_kernel<float, Spec<0, 2>> : (const void *)visc_rk_kernel<float, Spec<0, -1>>;
+        case 1: return z ? (const void *)visc_rk_kernel<float, Spec<1, 2>> : (const void *)visc_rk_kernel<float, Spec<1, -1>>;
+        case 2: return z ? (const void *)visc_rk_kernel<float, Spec<2, 2>> : (const void *)visc_rk_kernel<float, Spec<2, -1>>;
+        case 3: return z ? (const void *)visc_rk_kernel<float, Spec<3, 2>> : (const void *)visc_rk_kernel<float, Spec<3, -1>>;
+        default: return z ? (const void *)visc_rk_kernel<float, Spec<4, 2>> : (const void *)visc_rk_kernel<float, Spec<4, -1>>;
         }
+    } else {
+        return (const void *)visc_rk_kernel<T, RunSpec>;
     }
-    return (const void *)visc_rk_kernel<T, RunSpec>;
 }
 
 }  // namespace
@@ -144,11 +161,11 @@ cudaError_t init_visc_kernels()
     for (int ga = 0; ga < 3; ga += 2)
         for (int s = 0; s <= 4; ++s) {
             cudaError_t e = cudaFuncSetAttribute(visc_kernel_for<float>(s, ga),
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes<float>());
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)visc_smem<float>());
             if (e != cudaSuccess) return e;
         }
     return cudaFuncSetAttribute(visc_kernel_for<double>(0, 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)ring_bytes<double>());
+                                (int)visc_smem<double>());
 }
 
 template <typename T>
@@ -156,19 +173,9 @@ cudaError_t launch_visc_update(const BoxDev &bx, const T *W, const T *R, int sta
                                cudaStream_t st)
 {
     VArgs<T> a = make_vargs(bx, W, R, stage, g);
-    const int gx = (bx.n[0] + TX - 1) / TX, gy = (bx.n[1] + TY - 1) / TY;
-    // z chunk: enough blocks for the whole GPU, 8 to 32 planes per block (at
-    // 1024^3, 32 planes ran 1% faster than 64, a finer last wave; 16 paid
-    // more for the ring's start-up planes than it gained)
-    const long long want = 152LL * 8;
-    int nzc = (int)((want + (long long)gx * gy - 1) / ((long long)gx * gy));
-    int zc = (bx.n[2] + nzc - 1) / nzc;
-    if (zc < 8) zc = 8;
-    if (zc > 32) zc = 32;
-    a.zc = zc;
-    dim3 grid(gx, gy, (bx.n[2] + zc - 1) / zc);
+    const dim3 grid = visc_grid<T>(bx, a.zc);
     void *args[] = {&a};
-    return cudaLaunchKernel(visc_kernel_for<T>(stage, bx.ga), grid, dim3(TX * TY), args, ring_bytes<T>(), st);
+    return cudaLaunchKernel(visc_kernel_for<T>(stage, bx.ga), grid, dim3(VT), args, visc_smem<T>(), st);
 }
 
 template <typename T>
