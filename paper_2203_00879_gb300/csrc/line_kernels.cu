@@ -77,20 +77,16 @@ cudaError_t init_line_kernels()
 {
     cudaError_t e = cudaSuccess;
     cudaError_t r[] = {
-        allow_smem<float, MODE_FIELD, 0>(),  allow_smem<float, MODE_FIELD, 1>(),  allow_smem<float, MODE_FIELD, 2>(),
         allow_smem<double, MODE_FIELD, 0>(), allow_smem<double, MODE_FIELD, 1>(), allow_smem<double, MODE_FIELD, 2>(),
         allow_smem<double, MODE_FLUX, 0>(),  allow_smem<double, MODE_FLUX, 1>(),  allow_smem<double, MODE_FLUX, 2>(),
         allow_smem<double, MODE_FILTER, 0>(), allow_smem<double, MODE_FILTER, 1>(),
         allow_smem<double, MODE_FILTER, 2>(),  allow_smem<float, MODE_FILTER, 0>(),
         allow_smem<float, MODE_FILTER, 1>(),   allow_smem<float, MODE_FILTER, 2>(),
-        allow_smem<float, MODE_FIELD2, 0>(),   allow_smem<float, MODE_FIELD2, 1>(),
-        allow_smem<float, MODE_FIELD2, 2>(),   allow_smem<double, MODE_FIELD2, 0>(),
+        allow_smem<double, MODE_FIELD2, 0>(),
         allow_smem<double, MODE_FIELD2, 1>(),  allow_smem<double, MODE_FIELD2, 2>(),
-        allow_smem<float, MODE_VGRAD, 0>(),    allow_smem<float, MODE_VGRAD, 1>(),
-        allow_smem<float, MODE_VGRAD, 2>(),    allow_smem<double, MODE_VGRAD, 0>(),
+        allow_smem<double, MODE_VGRAD, 0>(),
         allow_smem<double, MODE_VGRAD, 1>(),   allow_smem<double, MODE_VGRAD, 2>(),
-        allow_smem<float, MODE_VDIV, 0>(),     allow_smem<float, MODE_VDIV, 1>(),
-        allow_smem<float, MODE_VDIV, 2>(),     allow_smem<double, MODE_VDIV, 0>(),
+        allow_smem<double, MODE_VDIV, 0>(),
         allow_smem<double, MODE_VDIV, 1>(),    allow_smem<double, MODE_VDIV, 2>()};
     for (cudaError_t x : r)
         if (x != cudaSuccess) e = x;
@@ -101,12 +97,23 @@ template <typename T>
 cudaError_t launch_line_field(const LineOpDev &op, int axis, const int n[3], const T *f, T *out,
                               double scale, cudaStream_t st)
 {
-    LineArgs<T> a{};
-    for (int d = 0; d < 3; ++d) a.n[d] = n[d];
-    a.in[0] = f;
-    a.out[0] = out;
-    a.scale = (T)scale;
-    return launch_any<T, MODE_FIELD>(op, axis, a, sizeof(T) == 4 ? 64 : 32, st);
+    if constexpr (sizeof(T) == 4) {
+        Sweep32Args a{};
+        if (!sweep32_operator(op, sweep_reach(MODE_FIELD), scale, a)) return cudaErrorInvalidValue;
+        a.in[0] = f;
+        a.out[0] = out;
+        sweep32_geometry(axis, n, a);
+        a.sub = op.sub;
+        a.nseg = op.nsub;
+        return launch_sweep32<MODE_FIELD>(axis, a, st);
+    } else {
+        LineArgs<T> a{};
+        for (int d = 0; d < 3; ++d) a.n[d] = n[d];
+        a.in[0] = f;
+        a.out[0] = out;
+        a.scale = (T)scale;
+        return launch_any<T, MODE_FIELD>(op, axis, a, 32, st);
+    }
 }
 
 template <typename T>
@@ -154,6 +161,17 @@ cudaError_t launch_line_filter(const LineOpDev &op, int axis, const BoxDev &bx, 
 cudaError_t launch_line_filter32(const LineOpDev &op, int axis, const BoxDev &bx, const float *in, float *out,
                                  cudaStream_t st)
 {
+    Sweep32Args s{};
+    if (sweep32_operator(op, sweep_reach(MODE_FILTER), 1.0, s)) {
+        for (int k = 0; k < 5; ++k) {
+            s.in[k] = in + (size_t)k * bx.np;
+            s.out[k] = out + (size_t)k * bx.np;
+        }
+        s.ga = bx.ga;
+        sweep32_geometry(axis, bx.n, s);
+        return launch_sweep32<MODE_FILTER>(axis, s, st);
+    }
+    // a coefficient near 1/2 couples farther than the recurrences' start-up
     LineArgs<float> a{};
     for (int d = 0; d < 3; ++d) a.n[d] = bx.n[d];
     for (int k = 0; k < 5; ++k) {
@@ -170,47 +188,77 @@ template <typename T>
 cudaError_t launch_line_field2(const LineOpDev &op, int axis, const int n[3], const T *f, T *out, double scale,
                                cudaStream_t st)
 {
-    LineArgs<T> a{};
-    for (int d = 0; d < 3; ++d) a.n[d] = n[d];
-    a.in[0] = f;
-    a.out[0] = out;
-    a.scale = (T)scale;
-    return launch_any<T, MODE_FIELD2>(op, axis, a, sizeof(T) == 4 ? 64 : 32, st);
+    if constexpr (sizeof(T) == 4) {
+        Sweep32Args a{};
+        if (!sweep32_operator(op, sweep_reach(MODE_FIELD2), scale, a)) return cudaErrorInvalidValue;
+        a.in[0] = f;
+        a.out[0] = out;
+        sweep32_geometry(axis, n, a);
+        a.sub = op.sub;
+        a.nseg = op.nsub;
+        return launch_sweep32<MODE_FIELD2>(axis, a, st);
+    } else {
+        LineArgs<T> a{};
+        for (int d = 0; d < 3; ++d) a.n[d] = n[d];
+        a.in[0] = f;
+        a.out[0] = out;
+        a.scale = (T)scale;
+        return launch_any<T, MODE_FIELD2>(op, axis, a, 32, st);
+    }
 }
 
 template <typename T>
 cudaError_t launch_line_vgrad(const LineOpDev &op, int axis, const BoxDev &bx, const T *W, T *G, cudaStream_t st)
 {
-    LineArgs<T> a{};
-    for (int d = 0; d < 3; ++d) a.n[d] = bx.n[d];
-    for (int k = 0; k < 5; ++k) a.in[k] = W + (size_t)k * bx.np;
-    for (int k = 0; k < 4; ++k) a.out[k] = G + (size_t)k * bx.np;
-    a.scale = (T)bx.inv_h[axis];
-    a.ga = bx.ga;
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 4) {
+        Sweep32Args a{};
+        if (!sweep32_operator(op, sweep_reach(MODE_VGRAD), bx.inv_h[axis], a)) return cudaErrorInvalidValue;
+        for (int k = 0; k < 5; ++k) a.in[k] = W + (size_t)k * bx.np;
+        for (int k = 0; k < 4; ++k) a.out[k] = G + (size_t)k * bx.np;
+        a.ga = bx.ga;
+        a.b0 = bx.T_b32;
+        a.b1 = bx.ip_b32;
+        a.b2 = bx.ir_b32;
+        sweep32_geometry(axis, bx.n, a);
+        return launch_sweep32<MODE_VGRAD>(axis, a, st);
+    } else {
+        LineArgs<T> a{};
+        for (int d = 0; d < 3; ++d) a.n[d] = bx.n[d];
+        for (int k = 0; k < 5; ++k) a.in[k] = W + (size_t)k * bx.np;
+        for (int k = 0; k < 4; ++k) a.out[k] = G + (size_t)k * bx.np;
+        a.scale = (T)bx.inv_h[axis];
+        a.ga = bx.ga;
         a.b0 = (const T *)bx.rho_b64;
         a.b1 = (const T *)bx.p_b64;
         a.gm2 = (T)bx.gm2;
-    } else {
-        a.b0 = (const T *)bx.T_b32;
-        a.b1 = (const T *)bx.ip_b32;
-        a.b2 = (const T *)bx.ir_b32;
+        return launch_any<T, MODE_VGRAD>(op, axis, a, 16, st);
     }
-    return launch_any<T, MODE_VGRAD>(op, axis, a, sizeof(T) == 4 ? 32 : 16, st);
 }
 
 template <typename T>
 cudaError_t launch_line_vdiv(const LineOpDev &op, int axis, const BoxDev &bx, const T *F, T *R, cudaStream_t st)
 {
-    LineArgs<T> a{};
-    for (int d = 0; d < 3; ++d) a.n[d] = bx.n[d];
-    for (int k = 0; k < 4; ++k) {
-        a.in[k] = F + (size_t)k * bx.np;
-        a.out[k] = R + (size_t)(1 + k) * bx.np;
+    if constexpr (sizeof(T) == 4) {
+        Sweep32Args a{};
+        if (!sweep32_operator(op, sweep_reach(MODE_VDIV), bx.inv_h[axis], a)) return cudaErrorInvalidValue;
+        for (int k = 0; k < 4; ++k) {
+            a.in[k] = F + (size_t)k * bx.np;
+            a.out[k] = R + (size_t)(1 + k) * bx.np;
+        }
+        a.ga = bx.ga;
+        sweep32_geometry(axis, bx.n, a);
+        return launch_sweep32<MODE_VDIV>(axis, a, st);
+    } else {
+        LineArgs<T> a{};
+        for (int d = 0; d < 3; ++d) a.n[d] = bx.n[d];
+        for (int k = 0; k < 4; ++k) {
+            a.in[k] = F + (size_t)k * bx.np;
+            a.out[k] = R + (size_t)(1 + k) * bx.np;
+        }
+        a.scale = (T)bx.inv_h[axis];
+        a.ga = bx.ga;
+        return launch_any<T, MODE_VDIV>(op, axis, a, 16, st);
     }
-    a.scale = (T)bx.inv_h[axis];
-    a.ga = bx.ga;
-    return launch_any<T, MODE_VDIV>(op, axis, a, sizeof(T) == 4 ? 32 : 16, st);
 }
 
 template cudaError_t launch_line_vgrad<float>(const LineOpDev &, int, const BoxDev &, const float *, float *,

@@ -28,7 +28,10 @@ enum LineMode { MODE_FIELD = 0, MODE_FLUX = 1, MODE_FILTER = 2, MODE_FIELD2 = 3,
 //   [10] lo, [11] hi         implicit rows solved by Thomas (lo > hi: none)
 //   [12] win_lo, [13] win_hi rows the solve reads (the end-row supports
 //                            outside them are consumed while staging)
-constexpr int SUB_REC = 14;
+//   [14], [15]             1 if the staged rows reach the line's first / last row
+//                            (true walls: a slab of a longer line keeps the
+//                            flags of the whole line)
+constexpr int SUB_REC = 16;
 
 // Host copy of a line operator (Sec. 3): partition, end rows, Thomas factors.
 struct LineOpHost {

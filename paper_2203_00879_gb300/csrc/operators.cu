@@ -312,6 +312,8 @@ bool build_line_op(int N, int sub_n, int kind, double alpha_f, double thresh, Li
         rec[3] = thi;
         rec[12] = wlo;
         rec[13] = whi;
+        rec[14] = tlo == 0;
+        rec[15] = thi == N - 1;
         int m = hi - lo + 1;
         if (m > op.maxm) op.maxm = m;
         if (thi - tlo + 1 > op.max_tile) op.max_tile = thi - tlo + 1;

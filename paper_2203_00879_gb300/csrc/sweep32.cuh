@@ -24,16 +24,22 @@
 //     alternating load, solve and store phases.
 //   scan_body (lines along x): a lane solves 8 consecutive points and takes
 //     the recurrences' state from its three neighbour lanes by shuffles.
-//     2.13 ms (44 B a point, 0.81 of the copy bandwidth; two thirds of the
+//     2.09 ms (44 B a point, 0.83 of the copy bandwidth; two thirds of the
 //     issue slots and three quarters of the shared-memory cycles used) against
 //     3.71 for whole lines in block-wide phases.
+// One field at 512^3 (8 B a point), x, y, z: 239, 240, 243 us against 469, 546,
+// 534 for the sub-domain tiles; compact viscous terms at 256^3, mean of the
+// axes: gradients 0.148 ms against 0.207, divergence 0.165 against 0.193.
 #pragma once
 
 #include "nopcs_internal.cuh"
 
 namespace nopcs {
 
-constexpr int SW_REACH = 24;  // rows after which the recurrences have forgotten their start (c^24 < 1e-8)
+// Rows after which the recurrences have forgotten their start (c^reach < 1e-8):
+// 24 for the first derivative (c = 0.46), 16 for the second derivative (0.19)
+// and the filter (0.14 at the paper's coefficient).
+constexpr int sweep_reach(int mode) { return mode == MODE_FILTER || mode == MODE_FIELD2 ? 16 : 24; }
 constexpr int SC_SHORT = 32;  // scan: lines shorter than this feel both walls
 constexpr int SC_P = 8;       // scan: points of a lane
 constexpr int SW_TAB = 20;    // rows tabulated next to a wall (the factors converge like c^(2r))
@@ -43,6 +49,7 @@ struct Sweep32Args {
     int N;                 // points of a line
     int cols, seg, nseg;   // march: lines, rows per segment, segments per line
     int ring;              // march: groups of a thread's ring (4 or 8)
+    const int *sub;        // march of a single field: sub-domain records (LineOpDev)
     int srow, sc;          // march: strides of a row and of the second line index
     int nch, tot;          // scan: 8-point chunks per line, chunks in all
     int kind;              // scan: 0 short lines, 1 single points, 2 four points a lane at a time
@@ -66,6 +73,7 @@ struct SweepMode {
     static constexpr bool SINGLE = MODE == MODE_FIELD || MODE == MODE_FIELD2;
     static constexpr int NF = SINGLE ? 1 : (MODE == MODE_VGRAD || MODE == MODE_VDIV ? 4 : 5);
     static constexpr int NIN = SINGLE ? 1 : (MODE == MODE_FLUX ? 6 : (MODE == MODE_VDIV ? 4 : 5));
+    static constexpr int REACH = sweep_reach(MODE);
     static constexpr int HW = MODE == MODE_FILTER ? 3 : 2;    // right-hand-side half-width
     static constexpr int NEXP = MODE == MODE_FILTER ? 3 : 2;  // explicit rows at a wall
     static constexpr int NB = MODE == MODE_FLUX ? 2 : (MODE == MODE_VGRAD ? 3 : 0);  // base tables used
@@ -130,10 +138,10 @@ __device__ __forceinline__ float sweep_rhs(const Sweep32Args &a, const float *w,
 constexpr int MARCH_TPB = 64;  // lines per block of a stand-alone march
 constexpr int SCAN_WARPS = 4;  // warps per block of a stand-alone scan
 
-// Host: the operator's coefficients with `scale` folded in (false if the
-// recurrences remember more than SW_REACH rows at 1e-8: a filter coefficient
+// Host: the operator's coefficients with `scale` folded in (false if its
+// recurrences remember more than `reach` rows at 1e-8: a filter coefficient
 // near 1/2), then the lines and pieces for a field of n points; a.N is set.
-bool sweep32_operator(const LineOpDev &op, double scale, Sweep32Args &a);
+bool sweep32_operator(const LineOpDev &op, int reach, double scale, Sweep32Args &a);
 void sweep32_geometry(int axis, const int n[3], Sweep32Args &a);
 // the convective sweep of a box along `axis`: R (= or -=) L(flux(W)) / h
 bool flux32_args(const LineOpDev &op, int axis, const BoxDev &bx, const float *W, float *R, Sweep32Args &a);
@@ -146,7 +154,13 @@ cudaError_t launch_sweep32(int axis, const Sweep32Args &a, cudaStream_t st);
 // thread.  When it is full, at group n, the backward recurrence starts at the
 // last row, runs back through groups n, n-1, n-2 (24 rows) and gives the final
 // values of the groups before them.  The inputs of the next group are in
-// flight meanwhile.
+// flight meanwhile.  (Where the reach is 16 rows, two groups of start-up do.)
+//
+// A sweep of a box cuts its lines where that fills the GPU.  A single field's
+// derivative cuts them at the sub-domains and reads nothing outside the rows
+// [tlo, thi] that a sub-domain's end rows reach (a row beyond repeats the last
+// one, 24 rows from any result): then a slab that holds these rows only gets
+// the bits of the whole line.
 constexpr int MR_G = 8;
 
 // shared memory of a march block
@@ -169,11 +183,21 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
     const int x = q % a.n[0], cc = q / a.n[0];
     const int base = x + cc * a.sc;
     const int N = a.N, srow = a.srow;
-    const int s = (int)(vblock % (unsigned)a.nseg) * a.seg, e = min(N, s + a.seg);
+    constexpr int LAG = M::REACH / MR_G;
+    const int seg = (int)(vblock % (unsigned)a.nseg);
     const int hrow = N - 1 - NEXP;  // last implicit row
-    const bool low = s == 0, high = e - 1 + SW_REACH >= hrow;
-    const int r0 = low ? 0 : s - SW_REACH;
-    const int G = ((high ? hrow : e - 1 + SW_REACH) - r0) / MR_G + 1;
+    int s, e, tlo = 0, thi = N - 1;
+    bool low, high;
+    if constexpr (M::SINGLE) {
+        const int *rec = a.sub + seg * SUB_REC;
+        s = rec[0], e = rec[1] + 1, tlo = rec[2], thi = rec[3];
+        low = rec[14] != 0, high = rec[15] != 0;
+    } else {
+        s = seg * a.seg, e = min(N, s + a.seg);
+        low = s == 0, high = e - 1 + M::REACH >= hrow;
+    }
+    const int r0 = low ? 0 : s - M::REACH;
+    const int G = ((high ? hrow : e - 1 + M::REACH) - r0) / MR_G + 1;
     int next = (s - r0) / MR_G;  // next group to give results
 
     const int kc = a.ga == 0 ? x : cc;  // coordinate along gravity (gravity not along the sweep)
@@ -212,6 +236,7 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
         if constexpr (NF > NV) d[NF - 1] = ring1[slot * TPB];
     };
     auto emit = [&](int row, const float *xv) {
+        if (M::SINGLE && (row < s || row >= e)) return;
         const int p = base + row * srow;
 #pragma unroll
         for (int k = 0; k < NF; ++k) {
@@ -228,13 +253,13 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
     float F[2 * HW + U][NF], v[U][NIN], dp[NF];
 #pragma unroll
     for (int u = 0; u < 2 * HW; ++u) {
-        const int row = min(max(r0 - HW + u, 0), N - 1);
+        const int row = min(max(r0 - HW + u, tlo), thi);
         float t[NIN];
         load(t, row);
         convert(t, row, F[u]);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) load(v[u], min(r0 + HW + u, N - 1));
+    for (int u = 0; u < U; ++u) load(v[u], min(max(r0 + HW + u, tlo), thi));
 #pragma unroll
     for (int k = 0; k < NF; ++k) dp[k] = 0.0f;
 #pragma unroll 1
@@ -246,13 +271,13 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
         for (int h = 0; h < MR_G / U; ++h) {
             const int ih = i0 + U * h, nx = ih + U + HW;  // nx: next step's first input row
 #pragma unroll
-            for (int u = 0; u < U; ++u) convert(v[u], min(ih + HW + u, N - 1), F[2 * HW + u]);
-            if (nx + U <= N) {
+            for (int u = 0; u < U; ++u) convert(v[u], min(ih + HW + u, thi), F[2 * HW + u]);
+            if (nx + U <= thi + 1 && (!M::SINGLE || nx >= tlo)) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) load(v[u], nx + u);
             } else if (h + 1 < MR_G / U || n + 1 < G) {
 #pragma unroll
-                for (int u = 0; u < U; ++u) load(v[u], min(nx + u, N - 1));
+                for (int u = 0; u < U; ++u) load(v[u], min(max(nx + u, tlo), thi));
             }
             if (FAST && (!low || i0 >= SW_TAB)) {
 #pragma unroll
@@ -295,9 +320,9 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
         // ---- backward, once R groups wait or the line ends ----
         const bool last = high && n == G - 1;
         if (n - next + 1 < R && n + 1 < G) continue;
-        if (n - 3 < next && !last) continue;
+        if (n - LAG < next && !last) continue;
         float X[NF];
-        int emax = i0 - 2 * MR_G;  // results: rows below emax
+        int emax = i0 - (LAG - 1) * MR_G;  // results: rows below emax
         if (last) {
             // explicit rows of the high wall, the last of which starts the
             // recurrence
@@ -336,7 +361,7 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
         }
         if (FAST && !last && (!low || next * MR_G >= SW_TAB)) {
 #pragma unroll 1
-            for (int m = n; m > n - 3; --m) {
+            for (int m = n; m > n - LAG; --m) {
 #pragma unroll
                 for (int u = MR_G - 1; u >= 0; --u) {
                     float d[NF];
@@ -346,7 +371,7 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
                 }
             }
 #pragma unroll 1
-            for (int m = n - 3; m >= next; --m) {
+            for (int m = n - LAG; m >= next; --m) {
 #pragma unroll
                 for (int u = MR_G - 1; u >= 0; --u) {
                     float d[NF];
@@ -372,7 +397,7 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
                 }
             }
         }
-        next = n - 2;
+        next = n - LAG + 1;
     }
 }
 
@@ -382,7 +407,7 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
 // lanes 3 .. 28 (three chunks are the 24 points the recurrences reach).  The
 // points are loaded and stored coalesced, 32 at a time, and change places
 // through a shared-memory tile that the warp has to itself.
-constexpr int SC_H = SW_REACH / SC_P;         // halo lanes on either side
+constexpr int SC_H = 3;                       // halo lanes on either side (24 points)
 constexpr int SC_USE = 32 - 2 * SC_H;         // lanes that give results
 constexpr int SC_FS = 4 + 8 * 36 + 4;         // floats of a field's tile: 32 points and 4 pad words, 8 times, halo words
 inline size_t scan_smem(int nf, int warps) { return (size_t)SC_FS * nf * warps * sizeof(float); }
@@ -427,6 +452,33 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
             if constexpr (NB > 2) bl[2] = a.b2[gk];
         }
     }
+    // SHORT: four more points on either side of the warp's (lanes 0 .. 3 load
+    // those before, lanes 4 .. 7 those after), for the end lanes' stencils.
+    // Longer lines leave the end lanes' outermost rows, which would need them,
+    // out of what they pass on (22 rows or more from a result).  Either way a
+    // result does not depend on where in a warp its chunk sits: equal lines
+    // give equal bits, and a slab's lines those of the whole box.
+    float eu[NIN];
+    float ey[3] = {0.0f, 0.0f, 0.0f};
+    bool ein = false;
+    if constexpr (SHORT) {
+        const int src = lane < 4 ? 0 : 31, d = lane < 4 ? lane - 4 : lane + 4;
+        const int A = __shfl_sync(ALL, addr, src), g = __shfl_sync(ALL, g0, src) + d, C = __shfl_sync(ALL, cnt, src);
+        ein = lane < 8 && C > 0 && g >= 0 && g < N;
+        const int p = ein ? A + d : addr;
+#pragma unroll
+        for (int m = 0; m < NIN; ++m) eu[m] = a.in[m][p];
+        if constexpr (NB > 0) {
+            const int ge = ein ? g : 0;
+#pragma unroll
+            for (int i = 0; i < NB; ++i) ey[i] = __shfl_sync(ALL, bl[i], src);
+            if (a.ga == 0) {
+                ey[0] = a.b0[ge];
+                ey[1] = a.b1[ge];
+                if constexpr (NB > 2) ey[2] = a.b2[ge];
+            }
+        }
+    }
 #pragma unroll
     for (int kb = 0; kb < KS; kb += KB) {
         float v[KB][NIN][E], bb[KB][E][3];
@@ -436,7 +488,7 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
             const int src = src_of(kb + k);
             const int A = __shfl_sync(ALL, addr, src), C = __shfl_sync(ALL, cnt, src);
             in[k] = el < C;
-            const int p = in[k] ? A + el : 0;  // the first points stand in for missing ones
+            const int p = in[k] ? A + el : A;  // a chunk's first points stand in for missing ones
 #pragma unroll
             for (int m = 0; m < NIN; ++m) {
                 if constexpr (VEC) {
@@ -486,20 +538,18 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
                 else
                     t[m * SC_FS] = f[0][m];
             }
-            // the halo words of the end lanes repeat the end points (their own
-            // results are not used)
-            if (kb + k == 0 && lane == 0) {
-#pragma unroll
-                for (int m = 0; m < NF; ++m)
-                    *reinterpret_cast<float4 *>(tile + m * SC_FS - 4) = make_float4(f[0][m], f[0][m], f[0][m], f[0][m]);
-            }
-            if (kb + k == KS - 1 && lane == 31) {
-#pragma unroll
-                for (int m = 0; m < NF; ++m)
-                    *reinterpret_cast<float4 *>(tile + m * SC_FS + 288) =
-                        make_float4(f[E - 1][m], f[E - 1][m], f[E - 1][m], f[E - 1][m]);
-            }
         }
+    }
+    if (lane < 8) {
+        float f[NF];
+#pragma unroll
+        for (int m = 0; m < NF; ++m) f[m] = 0.0f;
+        if constexpr (SHORT) {
+            if (ein) sweep_point<MODE, 0>(eu, ey, f);
+        }
+        float *const t = tile + (lane < 4 ? lane - 4 : 288 + lane - 4);
+#pragma unroll
+        for (int m = 0; m < NF; ++m) t[m * SC_FS] = f[m];
     }
     __syncwarp();
 
@@ -600,11 +650,19 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
                 }
             }
         }
+        // what a lane passes on to its third neighbour: without its outermost
+        // rows, whose stencils reach outside the lane
+        float dq = 0.0f, xq = 0.0f;
+        if constexpr (!SHORT) {
+            dq = d[HW];
+#pragma unroll
+            for (int j = HW + 1; j < P; ++j) dq = __fmaf_rn(-c, dq, d[j]);
+        }
 #pragma unroll
         for (int j = 1; j < P; ++j) d[j] = __fmaf_rn(SHORT ? -cp[j] : -c, d[j - 1], d[j]);
         {
             const float d1 = __shfl_up_sync(ALL, d[P - 1], 1), d2 = __shfl_up_sync(ALL, d[P - 1], 2),
-                        d3 = __shfl_up_sync(ALL, d[P - 1], 3);
+                        d3 = __shfl_up_sync(ALL, SHORT ? d[P - 1] : dq, 3);
             const float y = __fmaf_rn(wl[2], d3, __fmaf_rn(wl[1], d2, __fmul_rn(wl[0], d1)));
 #pragma unroll
             for (int j = 0; j < P; ++j) d[j] = __fmaf_rn(SHORT ? pf[j] : a.pw[j], y, d[j]);
@@ -617,11 +675,16 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
                 if (j > hj - (NEXP - 1)) d[j] = 0.0f;
             }
         }
+        if constexpr (!SHORT) {
+            xq = d[P - HW - 1];
+#pragma unroll
+            for (int j = P - HW - 2; j >= 0; --j) xq = __fmaf_rn(-c, xq, d[j]);
+        }
 #pragma unroll
         for (int j = P - 2; j >= 0; --j) d[j] = __fmaf_rn(SHORT ? -cp[j] : -c, d[j + 1], d[j]);
         {
             const float x1 = __shfl_down_sync(ALL, d[0], 1), x2 = __shfl_down_sync(ALL, d[0], 2),
-                        x3 = __shfl_down_sync(ALL, d[0], 3);
+                        x3 = __shfl_down_sync(ALL, SHORT ? d[0] : xq, 3);
             const float z = __fmaf_rn(wr[2], x3, __fmaf_rn(wr[1], x2, __fmul_rn(wr[0], x1)));
 #pragma unroll
             for (int j = 0; j < P; ++j) d[j] = __fmaf_rn(SHORT ? ps[j] : a.pw[P - 1 - j], z, d[j]);

@@ -41,17 +41,23 @@ cudaError_t launch_march_r(const Sweep32Args &a, cudaStream_t st)
 template <int MODE, int AXIS>
 cudaError_t launch_march(const Sweep32Args &a, cudaStream_t st)
 {
-    if (a.ring == 8) return launch_march_r<MODE, AXIS, 8, 32>(a, st);
-    return launch_march_r<MODE, AXIS, 4, 64>(a, st);
+    if constexpr (SweepMode<MODE>::SINGLE) {
+        // 512^3, sub-domains of 64, y and z: 240 and 243 us; a ring of 4 groups
+        // 234 and 248, but 48^3 8.3 us instead of 6.5
+        return launch_march_r<MODE, AXIS, 8, 64>(a, st);
+    } else {
+        if (a.ring == 8) return launch_march_r<MODE, AXIS, 8, 32>(a, st);
+        return launch_march_r<MODE, AXIS, 4, 64>(a, st);
+    }
 }
 
 }  // namespace
 
-bool sweep32_operator(const LineOpDev &op, double scale, Sweep32Args &a)
+bool sweep32_operator(const LineOpDev &op, int reach, double scale, Sweep32Args &a)
 {
     const double al = op.alpha;
     const double c = al == 0.0 ? 0.0 : (1.0 - sqrt(1.0 - 4.0 * al * al)) / (2.0 * al);
-    if (pow(fabs(c), SW_REACH) > 1e-8) return false;
+    if (pow(fabs(c), reach) > 1e-8) return false;
     const double inv = 1.0 / (1.0 - al * c);
     a.N = op.N;
     a.c = (float)c;
@@ -113,7 +119,7 @@ void sweep32_geometry(int axis, const int n[3], Sweep32Args &a)
 
 bool flux32_args(const LineOpDev &op, int axis, const BoxDev &bx, const float *W, float *R, Sweep32Args &a)
 {
-    if (!sweep32_operator(op, -bx.inv_h[axis], a)) return false;
+    if (!sweep32_operator(op, sweep_reach(MODE_FLUX), -bx.inv_h[axis], a)) return false;
     for (int k = 0; k < 6; ++k) a.in[k] = W + (size_t)k * bx.np;
     for (int k = 0; k < 5; ++k) a.out[k] = R + (size_t)k * bx.np;
     a.ga = bx.ga;
@@ -144,5 +150,10 @@ cudaError_t launch_sweep32(int axis, const Sweep32Args &a, cudaStream_t st)
 }
 
 template cudaError_t launch_sweep32<MODE_FLUX>(int, const Sweep32Args &, cudaStream_t);
+template cudaError_t launch_sweep32<MODE_FIELD>(int, const Sweep32Args &, cudaStream_t);
+template cudaError_t launch_sweep32<MODE_FIELD2>(int, const Sweep32Args &, cudaStream_t);
+template cudaError_t launch_sweep32<MODE_FILTER>(int, const Sweep32Args &, cudaStream_t);
+template cudaError_t launch_sweep32<MODE_VGRAD>(int, const Sweep32Args &, cudaStream_t);
+template cudaError_t launch_sweep32<MODE_VDIV>(int, const Sweep32Args &, cudaStream_t);
 
 }  // namespace nopcs

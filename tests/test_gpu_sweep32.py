@@ -51,3 +51,34 @@ def test_rhs_at_piece_ends(n, ga):
         assert np.all(err <= tol), (err / tol)
     finally:
         N.nopcs_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [(41, 6, 50), (65, 40, 9), (72, 33, 64), (24, 57, 30)])
+@pytest.mark.parametrize("order", [1, 3])
+def test_equal_lines_give_equal_bits(n, order):
+    """A field that varies along one axis only: every line along it has the bits
+    of the first, wherever its points fall in a warp or a block, and the FP32
+    result is within its rounding of the FP64 one (order 1: 32 ulps of max |f|
+    times the largest tap, 1.6 / h; order 3: 64 ulps times 4 / h^2)."""
+    import torch
+    N = binding()
+    p = S.box_params(n, sub_n=(16, 12, 24), perturb_amp=0.0)
+    ctx = N.nopcs_init([p], prec=N.NOPCS_MIXED, form=N.NOPCS_FORM_THOMAS, stream=stream_ptr())
+    try:
+        h = p["len"][0] / (n[0] - 1)
+        for axis in range(3):
+            v = np.random.default_rng(axis).uniform(0.5, 1.0, n[axis])
+            shape = [1, 1, 1]
+            shape[2 - axis] = n[axis]
+            f = np.broadcast_to(v.astype(np.float32).reshape(shape), n[::-1]).copy()
+            res = []
+            for dtype, fd in ((1, to_dev(f, np.float32)), (0, to_dev(f.astype(np.float64)))):
+                out = torch.empty_like(fd)
+                N.nopcs_derivative(ctx, 0, axis, order, dtype, fd.data_ptr(), out.data_ptr(), stream_ptr())
+                torch.cuda.synchronize()
+                res.append(np.moveaxis(out.cpu().numpy(), 2 - axis, -1).reshape(-1, n[axis]))
+            assert np.array_equal(res[0], np.broadcast_to(res[0][:1], res[0].shape)), axis
+            tol = 32 * 2.0 ** -24 * 1.6 / h if order == 1 else 64 * 2.0 ** -24 * 4.0 / h ** 2
+            assert np.abs(res[0][0] - res[1][0]).max() <= tol, axis
+    finally:
+        N.nopcs_destroy(ctx)
