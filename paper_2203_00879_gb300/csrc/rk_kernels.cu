@@ -47,8 +47,8 @@ __device__ __forceinline__ void prep_point(const BoxDev &bx, long long p, int kg
     } else {
         // deviation of the state from the hydrostatic base (mixed form), then
         // the primitives from it exactly as the stage kernels form them
-        const float D[5] = {(float)(r - bx.rho_b64[kg]), (float)mx, (float)my, (float)mz,
-                            (float)(E - bx.E_b64[kg])};
+        const float D[5] = {narrow_f64(r - bx.rho_b64[kg]), narrow_f64(mx), narrow_f64(my), narrow_f64(mz),
+                            narrow_f64(E - bx.E_b64[kg])};
         float Wv[6];
         prim_from_deviation(bx.rho_b32[kg], (float)(bx.gamma - 1.0), D, Wv);
 #pragma unroll
@@ -93,7 +93,7 @@ __global__ void filter_update_kernel(const BoxDev bx, double *__restrict__ Q, co
             double q[5];
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
-                q[k] = Q[k * np + p] + (double)(Fd[k * np + p] - Dn[k * np + p]);
+                q[k] = Q[k * np + p] + widen_f32(Fd[k * np + p] - Dn[k * np + p]);
                 Q[k * np + p] = q[k];
             }
             prep_point<float>(bx, p, kg, q[0], q[1], q[2], q[3], q[4], W, Dn);
@@ -199,7 +199,10 @@ __global__ void diag_partial_kernel(const BoxDev bx, const double *__restrict__ 
     // below only if its binary32 estimates, with margins well above their
     // rounding error, could reach the current maxima (or are not numbers);
     // the maxima are those of the FP64 values of the points that could raise
-    // them, so they are the same as evaluating every point in FP64
+    // them, so they are the same as evaluating every point in FP64.  The
+    // thresholds are those of the whole warp: a warp evaluates when any lane
+    // passes, so 32 lanes each finding maxima of their own kept it evaluating
+    // nearly every point of boxes up to 256^3
     float v5f = 0.0f, v6f = 0.0f, v7f = 0.0f;
     bool screening = true;
     int nseen = 0, ncand = 0;
@@ -216,71 +219,81 @@ __global__ void diag_partial_kernel(const BoxDev bx, const double *__restrict__ 
         // disturbances far smaller than p itself
         const double Eb_r = bx.ga != 0 && bx.E_b64 ? bx.E_b64[kr] : 0.0;
         const float cf_r = narrow_f64(gm1 * Eb_r - ph_r);
-        for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-            const long long p = base + x;
-            const double kgh = bx.ga == 0 ? x * bx.h[0] : kgh_r;
-            const double ph = bx.ga == 0 ? bx.p_h64[x] : ph_r;
-            const double r = Q[p], mx = Q[np + p], my = Q[2 * np + p], mz = Q[3 * np + p], E = Q[4 * np + p];
-            // not finite: exponent field all ones (infinity or NaN), tested on
-            // the high words by integer operations instead of FP64 compares
-            auto nonfinite = [](double q) { return ((unsigned)__double2hiint(q) & 0x7ff00000u) == 0x7ff00000u; };
-            const bool bad = nonfinite(r) || nonfinite(mx) || nonfinite(my) || nonfinite(mz) || nonfinite(E);
-            if (bad) v[8] = 1.0;
-            v[0] += r;
-            v[1] += mx;
-            v[2] += my;
-            v[3] += mz;
-            v[4] += E + r * bx.g * kgh;
-            // screen: |V|^2 to ~1e-6 relative; p to tol absolute (a few
-            // binary32 ulps of |E| + |kinetic| + |p_h|, with room to spare),
-            // so Mach^2 only where p is known to 1e-4 relative
-            bool cand = true;
-            if (screening) {
-                const double Eb = bx.ga == 0 ? (bx.E_b64 ? bx.E_b64[x] : 0.0) : Eb_r;
-                const float cf = bx.ga == 0 ? narrow_f64(gm1 * Eb - ph) : cf_r;
-                const float rf = narrow_f64(r), mxf = narrow_f64(mx), myf = narrow_f64(my), mzf = narrow_f64(mz);
-                const float Ef = narrow_f64(E), phf = narrow_f64(ph), dEf = narrow_f64(E - Eb);
-                const float irf = __fdividef(1.0f, rf);
-                const float s2f = (mxf * mxf + myf * myf + mzf * mzf) * (irf * irf);
-                const float kinf = 0.5f * rf * s2f;
-                const float prf = gm1f * (Ef - kinf);
-                const float tol = 2e-6f * (fabsf(Ef) + fabsf(kinf) + fabsf(phf));
-                // the disturbance pressure to 2e-6 of its own terms, plus 1e-14
-                // of E and p_h for the rounding of the FP64 evaluation it
-                // stands for
-                const float dpf = fabsf(gm1f * (dEf - kinf) + cf);
-                const float tol_dp =
-                    2e-6f * (fabsf(dEf) + fabsf(kinf) + fabsf(cf)) + 1e-14f * (fabsf(Ef) + fabsf(phf));
-                const float machf = __fdividef(s2f * rf * igamf, prf);
-                cand = !(s2f < v5f) || !(dpf + tol_dp < v6f) || !(fabsf(prf) > 1e4f * tol) ||
-                       !(machf * 1.0003f < v7f);
-                // a state whose maxima sit at the FP64 rounding floor (a box at
-                // rest) passes every point: the thread then stops screening
-                ncand += cand ? 1 : 0;
-                if (++nseen == 256) screening = 2 * ncand < nseen;
-            }
-            if (cand) {
-                const double ir = recip_newton(r);
-                const double u = mx * ir, vv = my * ir, w = mz * ir;
-                const double s2 = u * u + vv * vv + w * w;
-                const double pr = gm1 * (E - 0.5 * r * s2);
-                v[5] = fmax(v[5], s2);
-                v[6] = fmax(v[6], fabs(pr - ph));
-                // Mach^2 = num / pr can raise the maximum only where num
-                // exceeds v7 pr (for pr > 0; the factor 0.999999 keeps every
-                // point whose rounded quotient could exceed v7).  Elsewhere the
-                // quotient is at most v7, or not a number, and the maximum
-                // stays as it is.
-                const double num = s2 * r * igam;
-                if (num > v7t * pr) {
-                    v[7] = fmax(v[7], num / pr);
-                    v7t = v[7] * 0.999999;
+        for (int xw = threadIdx.x & ~31; xw < nx; xw += blockDim.x) {
+            const int x = xw + (int)(threadIdx.x & 31);
+            bool cand = false;
+            if (x < nx) {
+                const long long p = base + x;
+                const double kgh = bx.ga == 0 ? x * bx.h[0] : kgh_r;
+                const double ph = bx.ga == 0 ? bx.p_h64[x] : ph_r;
+                const double r = Q[p], mx = Q[np + p], my = Q[2 * np + p], mz = Q[3 * np + p], E = Q[4 * np + p];
+                // not finite: exponent field all ones (infinity or NaN), tested on
+                // the high words by integer operations instead of FP64 compares
+                auto nonfinite = [](double q) { return ((unsigned)__double2hiint(q) & 0x7ff00000u) == 0x7ff00000u; };
+                const bool bad = nonfinite(r) || nonfinite(mx) || nonfinite(my) || nonfinite(mz) || nonfinite(E);
+                if (bad) v[8] = 1.0;
+                v[0] += r;
+                v[1] += mx;
+                v[2] += my;
+                v[3] += mz;
+                v[4] += E + r * bx.g * kgh;
+                // screen: |V|^2 to ~1e-6 relative; p to tol absolute (a few
+                // binary32 ulps of |E| + |kinetic| + |p_h|, with room to spare),
+                // so Mach^2 only where p is known to 1e-4 relative
+                cand = true;
+                if (screening) {
+                    const double Eb = bx.ga == 0 ? (bx.E_b64 ? bx.E_b64[x] : 0.0) : Eb_r;
+                    const float cf = bx.ga == 0 ? narrow_f64(gm1 * Eb - ph) : cf_r;
+                    const float rf = narrow_f64(r), mxf = narrow_f64(mx), myf = narrow_f64(my), mzf = narrow_f64(mz);
+                    const float Ef = narrow_f64(E), phf = narrow_f64(ph), dEf = narrow_f64(E - Eb);
+                    const float irf = __fdividef(1.0f, rf);
+                    const float s2f = (mxf * mxf + myf * myf + mzf * mzf) * (irf * irf);
+                    const float kinf = 0.5f * rf * s2f;
+                    const float prf = gm1f * (Ef - kinf);
+                    const float tol = 2e-6f * (fabsf(Ef) + fabsf(kinf) + fabsf(phf));
+                    // the disturbance pressure to 2e-6 of its own terms, plus 1e-14
+                    // of E and p_h for the rounding of the FP64 evaluation it
+                    // stands for
+                    const float dpf = fabsf(gm1f * (dEf - kinf) + cf);
+                    const float tol_dp =
+                        2e-6f * (fabsf(dEf) + fabsf(kinf) + fabsf(cf)) + 1e-14f * (fabsf(Ef) + fabsf(phf));
+                    const float machf = __fdividef(s2f * rf * igamf, prf);
+                    cand = !(s2f < v5f) || !(dpf + tol_dp < v6f) || !(fabsf(prf) > 1e4f * tol) ||
+                           !(machf * 1.0003f < v7f);
+                    // a state whose maxima sit at the FP64 rounding floor (a box at
+                    // rest) passes every point: the thread then stops screening
+                    ncand += cand ? 1 : 0;
+                    if (++nseen == 256) screening = 2 * ncand < nseen;
                 }
-                // thresholds a little below the maxima; none while a maximum is
-                // too small for the binary32 estimates to resolve
-                v5f = v[5] > 1e-30 ? narrow_f64(v[5]) * 0.99999f : 0.0f;
-                v6f = narrow_f64(v[6]) * 0.99999f;
-                v7f = v[7] > 1e-30 ? narrow_f64(v[7]) * 0.9999f : 0.0f;
+                if (cand) {
+                    const double ir = recip_newton(r);
+                    const double u = mx * ir, vv = my * ir, w = mz * ir;
+                    const double s2 = u * u + vv * vv + w * w;
+                    const double pr = gm1 * (E - 0.5 * r * s2);
+                    v[5] = fmax(v[5], s2);
+                    v[6] = fmax(v[6], fabs(pr - ph));
+                    // Mach^2 = num / pr can raise the maximum only where num
+                    // exceeds v7 pr (for pr > 0; the factor 0.999999 keeps every
+                    // point whose rounded quotient could exceed v7).  Elsewhere the
+                    // quotient is at most v7, or not a number, and the maximum
+                    // stays as it is.
+                    const double num = s2 * r * igam;
+                    if (num > v7t * pr) {
+                        v[7] = fmax(v[7], num / pr);
+                        v7t = v[7] * 0.999999;
+                    }
+                }
+            }
+            if (__any_sync(0xffffffffu, cand)) {
+                // thresholds a little below the warp's maxima (not negative, so
+                // their bit patterns are ordered as the values are); none while
+                // a maximum is too small for the binary32 estimates to resolve
+                auto warp_max = [](float f) {
+                    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(f)));
+                };
+                v5f = warp_max(v[5] > 1e-30 ? narrow_f64(v[5]) * 0.99999f : 0.0f);
+                v6f = warp_max(narrow_f64(v[6]) * 0.99999f);
+                v7f = warp_max(v[7] > 1e-30 ? narrow_f64(v[7]) * 0.9999f : 0.0f);
             }
         }
     }
