@@ -2,7 +2,7 @@
 //
 // A box's RK4 step is a chain of phases -- per stage the x, y and z flux
 // sweeps (Sec. 3), the fused viscous / source / RK kernel (Sec. 2, Sec. 4) and
-// the wall conditions (faces, then edges and corners) -- and each phase is a
+// the wall conditions -- and each phase is a
 // set of independent blocks: the blocks the stand-alone kernels would launch.
 // Here one kernel runs them all.  The host lists work items (box, stage,
 // phase, a run of blocks), each box's phases in order; every block of the
@@ -39,11 +39,11 @@ constexpr int BT = 256;             // threads per block (the viscous tile's)
 // with 160 lines and 8 rows 42.2 and 10.7, at three blocks per SM (80 registers
 // a thread, the sweeps spill) with 96 lines and 2 rows 46.5 and 11.6.
 constexpr int BMARCH = 128, BU = 4;
-// wall nodes per tile of the face and edge phases: four passes of a block,
-// so that a box's wall phases spread over many blocks instead of holding the
-// box's next phase behind a few long items
-constexpr int WALL_CHUNK = 4 * BT;
-enum { PH_SX = 0, PH_SY, PH_SZ, PH_VISC, PH_FACE, PH_EDGE, PH_CORNER, NPH };
+// wall nodes per tile: four passes of a block, so that a box's wall phase
+// spreads over many blocks instead of holding the box's next phase behind a few
+// long items
+constexpr unsigned WALL_CHUNK = 4 * BT;
+enum { PH_SX = 0, PH_SY, PH_SZ, PH_VISC, PH_WALL, PH_CORNER, NPH };
 
 struct BStage {
     Sweep32Args sw[3];
@@ -226,32 +226,14 @@ __global__ void __launch_bounds__(BT, 2) batch_step_kernel(const BParams p)
                 case PH_SY: run_march<1>(*ssw, v, reinterpret_cast<float *>(smraw)); break;
                 case PH_SZ: run_march<2>(*ssw, v, reinterpret_cast<float *>(smraw)); break;
                 case PH_VISC: run_visc_any(*sva, v % B.gx, (v / B.gx) % B.gy, v / (B.gx * B.gy), smraw); break;
-                case PH_FACE: {
-                    const long long tot = face_count(B.bx);
-                    const long long t1 = min(tot, (long long)(v + 1) * WALL_CHUNK);
-                    for (long long t = (long long)v * WALL_CHUNK + threadIdx.x; t < t1; t += BT) {
-                        int c[3];
-                        face_node(B.bx, t, c);
-                        wall_node(B.bx, c, S.Q, S.Dn, S.Wf, S.Ww);
-                    }
-                    break;
-                }
-                case PH_EDGE: {
-                    const long long tot = edge_count(B.bx);
-                    const long long t1 = min(tot, (long long)(v + 1) * WALL_CHUNK);
-                    for (long long t = (long long)v * WALL_CHUNK + threadIdx.x; t < t1; t += BT) {
-                        int c[3];
-                        edge_node(B.bx, t, c);
-                        wall_node(B.bx, c, S.Q, S.Dn, S.Wf, S.Ww);
-                    }
+                case PH_WALL: {
+                    const unsigned t1 = min(wall_count(B.bx), (unsigned)(v + 1) * WALL_CHUNK);
+                    for (unsigned t = (unsigned)v * WALL_CHUNK + threadIdx.x; t < t1; t += BT)
+                        wall_node(B.bx, t, S.Q, S.Dn, S.Wf, S.Ww);
                     break;
                 }
                 default: {  // the corners, which read the edges
-                    if (threadIdx.x < 8) {
-                        int c[3];
-                        corner_node(B.bx, threadIdx.x, c);
-                        wall_node(B.bx, c, S.Q, S.Dn, S.Wf, S.Ww);
-                    }
+                    if (threadIdx.x < 8) corner_node(B.bx, threadIdx.x, S.Q, S.Dn, S.Wf, S.Ww);
                 }
                 }
                 __syncthreads();  // the next block of the item reuses the shared memory
@@ -326,11 +308,7 @@ cudaError_t batch_plan_build(const std::vector<BatchBoxIn> &in, BatchPlan **out,
                 S.Ww = nullptr;
             }
         }
-        const long long nface = 2 * ((long long)(I.bx.n[1] - 2) * (I.bx.n[2] - 2) +
-                                     (long long)(I.bx.n[0] - 2) * (I.bx.n[2] - 2) +
-                                     (long long)(I.bx.n[0] - 2) * (I.bx.n[1] - 2));
-        B.ntile[PH_FACE] = (int)((nface + WALL_CHUNK - 1) / WALL_CHUNK);
-        B.ntile[PH_EDGE] = (int)((edge_count(I.bx) + WALL_CHUNK - 1) / WALL_CHUNK);
+        B.ntile[PH_WALL] = (int)((wall_count(I.bx) + WALL_CHUNK - 1) / WALL_CHUNK);
         B.ntile[PH_CORNER] = 1;
         // blocks per item: about a quarter of a GPU wave per phase of a big
         // box, single blocks for small ones

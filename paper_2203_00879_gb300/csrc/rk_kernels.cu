@@ -101,35 +101,16 @@ __global__ void filter_update_kernel(const BoxDev bx, double *__restrict__ Q, co
     }
 }
 
-__global__ void wall_face_kernel(const BoxDev bx, double *Q, float *Dn, float *Wf, float *Ww)
+__global__ void wall_kernel(const BoxDev bx, double *Q, float *Dn, float *Wf, float *Ww)
 {
-    const long long tot = face_count(bx);
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x) {
-        int c[3];
-        face_node(bx, t, c);
-        wall_node(bx, c, Q, Dn, Wf, Ww);
-    }
-}
-
-__global__ void wall_edge_kernel(const BoxDev bx, double *Q, float *Dn, float *Wf, float *Ww)
-{
-    const long long tot = edge_count(bx);
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x) {
-        int c[3];
-        edge_node(bx, t, c);
-        wall_node(bx, c, Q, Dn, Wf, Ww);
-    }
+    const unsigned tot = wall_count(bx);
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += gridDim.x * blockDim.x)
+        wall_node(bx, t, Q, Dn, Wf, Ww);
 }
 
 __global__ void wall_corner_kernel(const BoxDev bx, double *Q, float *Dn, float *Wf, float *Ww)
 {
-    if (threadIdx.x < 8) {
-        int c[3];
-        corner_node(bx, threadIdx.x, c);
-        wall_node(bx, c, Q, Dn, Wf, Ww);
-    }
+    if (threadIdx.x < 8) corner_node(bx, threadIdx.x, Q, Dn, Wf, Ww);
 }
 
 // ---------------------------------------------------------------------------
@@ -372,14 +353,8 @@ cudaError_t launch_filter_update(const BoxDev &bx, double *Q, const float *Fd, f
 
 cudaError_t launch_wall_bc(const BoxDev &bx, double *Q, float *Dn, float *Wf, float *Ww, cudaStream_t st)
 {
-    const long long faces = 2LL * ((long long)(bx.n[1] - 2) * (bx.n[2] - 2) + (long long)(bx.n[0] - 2) * (bx.n[2] - 2) +
-                                   (long long)(bx.n[0] - 2) * (bx.n[1] - 2));
-    wall_face_kernel<<<grid_for(faces, 256), 256, 0, st>>>(bx, Q, Dn, Wf, Ww);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long long edges = 4LL * ((bx.n[0] - 2) + (bx.n[1] - 2) + (bx.n[2] - 2));
-    wall_edge_kernel<<<grid_for(edges, 256), 256, 0, st>>>(bx, Q, Dn, Wf, Ww);
-    e = cudaGetLastError();
+    wall_kernel<<<grid_for(wall_count(bx), 128), 128, 0, st>>>(bx, Q, Dn, Wf, Ww);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     wall_corner_kernel<<<1, 32, 0, st>>>(bx, Q, Dn, Wf, Ww);
     return cudaGetLastError();

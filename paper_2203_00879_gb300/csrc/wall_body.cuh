@@ -12,173 +12,240 @@ namespace {
 // ---------------------------------------------------------------------------
 // No-slip adiabatic walls: momentum zero on every wall node (kept by the
 // update), T_w = (4 T_1 - T_2) / 3 along the inward normal, averaged over the
-// normals of edge and corner nodes; faces first, then edges from the faces,
-// then corners from the edges.  E_w = rho_w T_w / (gamma (gamma-1) M^2).
+// normals of edge and corner nodes, where T_1 and T_2 are wall temperatures
+// themselves (edges from the faces, corners from the edges).
+// E_w = rho_w T_w / (gamma (gamma-1) M^2).
+//
+// Faces and edges are set in one pass: an edge node works out the four face
+// temperatures it needs from the four interior nodes behind them instead of
+// waiting for them, so nothing reads what another thread writes (the density of
+// a wall node is not written).  The corners follow, from the stored edges.
+// Bound by latency at all but the largest sizes: every load of a node is issued
+// before its first use.  Faces, edges and corners as three launches with
+// branches between the loads: 31 us per stage in boxes of 32 to 128 points, now
+// 22; 256^3 70 us, now 57.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double temp_q(const BoxDev &bx, const double *Q, long long i)
-{
-    const long long np = bx.np;
-    const double r = Q[i];
-    const double ke = 0.5 * (Q[np + i] * Q[np + i] + Q[2 * np + i] * Q[2 * np + i] + Q[3 * np + i] * Q[3 * np + i]) / r;
-    return bx.gm2 * (bx.gamma - 1.0) * (Q[4 * np + i] - ke) / r;
-}
 
-__device__ void set_wall_node(const BoxDev &bx, double *Q, const int c[3], float *Dn, float *Wf)
-{
-    const long long st[3] = {1, bx.n[0], (long long)bx.n[0] * bx.n[1]};
-    const long long i = c[0] + st[1] * c[1] + st[2] * c[2];
-    double Tw = 0.0;
-    int nw = 0;
-    for (int d = 0; d < 3; ++d) {
-        long long s;
-        if (c[d] == 0)
-            s = st[d];
-        else if (c[d] == bx.n[d] - 1)
-            s = -st[d];
-        else
-            continue;
-        Tw += (4.0 * temp_q(bx, Q, i + s) - temp_q(bx, Q, i + 2 * s)) / 3.0;
-        ++nw;
+// On the FP64 state (refreshing D_n and W when given).  A value is a
+// temperature.
+struct WallState {
+    using T = double;
+    const BoxDev &bx;
+    double *Q;
+    float *Dn, *Wf;
+    __device__ __forceinline__ double temp(double r, double mx, double my, double mz, double E) const
+    {
+        const double ke = 0.5 * (mx * mx + my * my + mz * mz) / r;
+        return bx.gm2 * (bx.gamma - 1.0) * (E - ke) / r;
     }
-    Tw /= nw;
-    const long long np = bx.np;
-    Q[np + i] = Q[2 * np + i] = Q[3 * np + i] = 0.0;
-    Q[4 * np + i] = Q[i] * Tw * bx.cE;
-    if (Dn) {
-        const int kg = c[bx.ga];
-        const float D[5] = {(float)(Q[i] - bx.rho_b64[kg]), 0.0f, 0.0f, 0.0f, (float)(Q[4 * np + i] - bx.E_b64[kg])};
-        float Wv[6];
-        prim_from_deviation(bx.rho_b32[kg], (float)(bx.gamma - 1.0), D, Wv);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) Dn[k * np + i] = D[k];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) Wf[k * np + i] = Wv[k];
+    // value of a stored node
+    __device__ __forceinline__ double node(long long i, int) const
+    {
+        const long long np = bx.np;
+        return temp(Q[i], Q[np + i], Q[2 * np + i], Q[3 * np + i], Q[4 * np + i]);
     }
-}
-
-// ---------------------------------------------------------------------------
-// The same wall conditions on an FP32 stage state held as W (mixed form):
-// T = T_b + T' with T' = T_b (p'/p_b - rho'/rho_b) / (1 + rho'/rho_b), the
-// extrapolated wall temperature kept as its difference dT from T_b at the
-// node, and E_w - E_b = cE (rho' T_w + rho_b dT) (E_b = cE rho_b T_b).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ float temp_dev_w(const BoxDev &bx, const float *W, long long i, int kg)
-{
-    const long long np = bx.np;
-    const float rr = W[i] * bx.ir_b32[kg];
-    return bx.T_b32[kg] * (W[4 * np + i] * bx.ip_b32[kg] - rr) / (1.0f + rr);
-}
-
-__device__ void set_wall_node_w(const BoxDev &bx, float *W, const int c[3])
-{
-    const long long st[3] = {1, bx.n[0], (long long)bx.n[0] * bx.n[1]};
-    const long long i = c[0] + st[1] * c[1] + st[2] * c[2];
-    const int kg = c[bx.ga];
-    const float TbP = bx.T_b32[kg];
-    float dT = 0.0f;
-    int nw = 0;
-    for (int d = 0; d < 3; ++d) {
-        int sg;
-        if (c[d] == 0)
-            sg = 1;
-        else if (c[d] == bx.n[d] - 1)
-            sg = -1;
-        else
-            continue;
-        const long long s = sg * st[d];
-        int k1 = kg, k2 = kg;
-        if (d == bx.ga) {
-            k1 = kg + sg;
-            k2 = kg + 2 * sg;
+    // extrapolation to a wall node from the nodes one and two inside
+    __device__ __forceinline__ double extrapolate(int, int, double t1, int, double t2) const
+    {
+        return (4.0 * t1 - t2) / 3.0;
+    }
+    // value of a wall node that extrapolates to tw (through the energy it stores)
+    __device__ __forceinline__ double wall(long long i, int, double tw) const
+    {
+        const double r = Q[i];
+        return temp(r, 0.0, 0.0, 0.0, r * tw * bx.cE);
+    }
+    __device__ __forceinline__ void store(long long i, int kg, double tw) const
+    {
+        const long long np = bx.np;
+        const double r = Q[i], E = r * tw * bx.cE;
+        Q[np + i] = Q[2 * np + i] = Q[3 * np + i] = 0.0;
+        Q[4 * np + i] = E;
+        if (Dn) {
+            const float Dv[5] = {(float)(r - bx.rho_b64[kg]), 0.0f, 0.0f, 0.0f, (float)(E - bx.E_b64[kg])};
+            float Wv[6];
+            prim_from_deviation(bx.rho_b32[kg], (float)(bx.gamma - 1.0), Dv, Wv);
+#pragma unroll
+            for (int k = 0; k < 5; ++k) Dn[k * np + i] = Dv[k];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) Wf[k * np + i] = Wv[k];
         }
-        const float d1 = (bx.T_b32[k1] - TbP) + temp_dev_w(bx, W, i + s, k1);
-        const float d2 = (bx.T_b32[k2] - TbP) + temp_dev_w(bx, W, i + 2 * s, k2);
-        dT += (4.0f * d1 - d2) * (1.0f / 3.0f);
-        ++nw;
     }
-    dT /= (float)nw;
-    const long long np = bx.np;
-    const float rd = W[i];
-    const float Ed = (float)bx.cE * (rd * (TbP + dT) + bx.rho_b32[kg] * dT);
-    const float pd = (float)(bx.gamma - 1.0) * Ed;
-    W[np + i] = W[2 * np + i] = W[3 * np + i] = 0.0f;
-    W[4 * np + i] = pd;
-    W[5 * np + i] = Ed + pd;
+};
+
+// On an FP32 stage state held as W (mixed form).  A node's value is T' of T =
+// T_b + T', T' = T_b (p'/p_b - rho'/rho_b) / (1 + rho'/rho_b); an extrapolated
+// wall temperature is its difference dT from T_b at the wall node, and
+// E_w - E_b = cE (rho' T_w + rho_b dT) (E_b = cE rho_b T_b).
+struct WallStage {
+    using T = float;
+    const BoxDev &bx;
+    float *W;
+    __device__ __forceinline__ float dtemp(float rd, float pd, int kg) const
+    {
+        const float rr = rd * bx.ir_b32[kg];
+        return bx.T_b32[kg] * (pd * bx.ip_b32[kg] - rr) / (1.0f + rr);
+    }
+    __device__ __forceinline__ float energy(float rd, int kg, float dT) const
+    {
+        return (float)bx.cE * (rd * (bx.T_b32[kg] + dT) + bx.rho_b32[kg] * dT);
+    }
+    __device__ __forceinline__ float node(long long i, int kg) const { return dtemp(W[i], W[4 * bx.np + i], kg); }
+    __device__ __forceinline__ float extrapolate(int kg, int k1, float t1, int k2, float t2) const
+    {
+        const float TbP = bx.T_b32[kg];
+        const float d1 = (bx.T_b32[k1] - TbP) + t1, d2 = (bx.T_b32[k2] - TbP) + t2;
+        return (4.0f * d1 - d2) * (1.0f / 3.0f);
+    }
+    __device__ __forceinline__ float wall(long long i, int kg, float dT) const
+    {
+        const float rd = W[i];
+        return dtemp(rd, (float)(bx.gamma - 1.0) * energy(rd, kg, dT), kg);
+    }
+    __device__ __forceinline__ void store(long long i, int kg, float dT) const
+    {
+        const long long np = bx.np;
+        const float Ed = energy(W[i], kg, dT);
+        const float pd = (float)(bx.gamma - 1.0) * Ed;
+        W[np + i] = W[2 * np + i] = W[3 * np + i] = 0.0f;
+        W[4 * np + i] = pd;
+        W[5 * np + i] = Ed + pd;
+    }
+};
+
+// One step inwards along axis d from a node with coordinate c there: in the
+// node index and in the coordinate along gravity.
+struct Inward {
+    long long s;
+    int k;
+    __device__ __forceinline__ Inward(const BoxDev &bx, int d, int c)
+    {
+        const int sg = c == 0 ? 1 : -1;
+        s = sg * (d == 0 ? 1LL : (d == 1 ? (long long)bx.n[0] : (long long)bx.n[0] * bx.n[1]));
+        k = d == bx.ga ? sg : 0;
+    }
+};
+
+template <class S>
+__device__ __forceinline__ typename S::T along(const S &w, long long i, int kg, const Inward &d)
+{
+    const auto t1 = w.node(i + d.s, kg + d.k), t2 = w.node(i + 2 * d.s, kg + 2 * d.k);
+    return w.extrapolate(kg, kg + d.k, t1, kg + 2 * d.k, t2);
+}
+template <class S>
+__device__ __forceinline__ void face_update(const S &w, long long i, int kg, const Inward &d)
+{
+    w.store(i, kg, along(w, i, kg, d));
+}
+// a, b: the edge's two normals, in the order of their axes
+template <class S>
+__device__ __forceinline__ void edge_update(const S &w, long long i, int kg, const Inward &a, const Inward &b)
+{
+    using T = typename S::T;
+    T t[2][2];  // interior nodes, steps along a and b
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) t[p][q] = w.node(i + (p + 1) * a.s + (q + 1) * b.s, kg + (p + 1) * a.k + (q + 1) * b.k);
+    T fa[2], fb[2];  // the face nodes along a (on the wall of b) and along b
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const int ka = kg + (p + 1) * a.k, kb = kg + (p + 1) * b.k;
+        fa[p] = w.wall(i + (p + 1) * a.s, ka, w.extrapolate(ka, ka + b.k, t[p][0], ka + 2 * b.k, t[p][1]));
+        fb[p] = w.wall(i + (p + 1) * b.s, kb, w.extrapolate(kb, kb + a.k, t[0][p], kb + 2 * a.k, t[1][p]));
+    }
+    w.store(i, kg, (w.extrapolate(kg, kg + a.k, fa[0], kg + 2 * a.k, fa[1]) +
+                    w.extrapolate(kg, kg + b.k, fb[0], kg + 2 * b.k, fb[1])) / T(2));
 }
 
-// face nodes: exactly one wall coordinate; node t of 2 (fx + fy + fz)
-__host__ __device__ __forceinline__ long long face_count(const BoxDev &bx)
+// Wall nodes in order: faces (one wall coordinate), edges (two).
+// A box of fewer than 2^31 points has fewer than 2^31 of them.
+__host__ __device__ __forceinline__ unsigned face_count(const BoxDev &bx)
 {
-    const long long nx = bx.n[0], ny = bx.n[1], nz = bx.n[2];
-    return 2 * ((ny - 2) * (nz - 2) + (nx - 2) * (nz - 2) + (nx - 2) * (ny - 2));
+    const unsigned nx = bx.n[0] - 2, ny = bx.n[1] - 2, nz = bx.n[2] - 2;
+    return 2u * (ny * nz + nx * nz + nx * ny);
 }
-__device__ __forceinline__ void face_node(const BoxDev &bx, long long t, int c[3])
+__host__ __device__ __forceinline__ unsigned edge_count(const BoxDev &bx)
 {
-    const int nx = bx.n[0], ny = bx.n[1], nz = bx.n[2];
-    const long long fx = (long long)(ny - 2) * (nz - 2), fy = (long long)(nx - 2) * (nz - 2),
-                    fz = (long long)(nx - 2) * (ny - 2);
-    long long q = t;
-    if (q < 2 * fx) {
-        int side = (int)(q / fx);
-        q %= fx;
-        c[0] = side ? nx - 1 : 0;
-        c[1] = 1 + (int)(q % (ny - 2));
-        c[2] = 1 + (int)(q / (ny - 2));
-    } else if ((q -= 2 * fx) < 2 * fy) {
-        int side = (int)(q / fy);
-        q %= fy;
-        c[1] = side ? ny - 1 : 0;
-        c[0] = 1 + (int)(q % (nx - 2));
-        c[2] = 1 + (int)(q / (nx - 2));
-    } else {
-        q -= 2 * fy;
-        int side = (int)(q / fz);
-        q %= fz;
-        c[2] = side ? nz - 1 : 0;
-        c[0] = 1 + (int)(q % (nx - 2));
-        c[1] = 1 + (int)(q / (nx - 2));
+    return 4u * (unsigned)(bx.n[0] - 2 + bx.n[1] - 2 + bx.n[2] - 2);
+}
+// faces and edges
+__host__ __device__ __forceinline__ unsigned wall_count(const BoxDev &bx)
+{
+    return face_count(bx) + edge_count(bx);
+}
+// wall node t (a face or an edge node) of the state seen through w
+template <class S>
+__device__ __forceinline__ void wall_update(const BoxDev &bx, unsigned q, const S &w)
+{
+    const unsigned m[3] = {(unsigned)bx.n[0] - 2u, (unsigned)bx.n[1] - 2u, (unsigned)bx.n[2] - 2u};
+    int c[3] = {0, 0, 0};
+    const unsigned fx = m[1] * m[2], fy = m[0] * m[2], fz = m[0] * m[1];
+    auto at = [&] { return c[0] + (long long)bx.n[0] * (c[1] + (long long)bx.n[1] * c[2]); };
+    auto kg = [&] { return bx.ga == 0 ? c[0] : (bx.ga == 1 ? c[1] : c[2]); };
+    if (q < 2u * (fx + fy + fz)) {
+        int d;
+        if (q < 2u * fx) {
+            const unsigned side = q >= fx, r = q - side * fx;
+            c[0] = side ? bx.n[0] - 1 : 0, c[1] = 1 + (int)(r % m[1]), c[2] = 1 + (int)(r / m[1]);
+            d = 0;
+        } else if ((q -= 2u * fx) < 2u * fy) {
+            const unsigned side = q >= fy, r = q - side * fy;
+            c[1] = side ? bx.n[1] - 1 : 0, c[0] = 1 + (int)(r % m[0]), c[2] = 1 + (int)(r / m[0]);
+            d = 1;
+        } else {
+            q -= 2u * fy;
+            const unsigned side = q >= fz, r = q - side * fz;
+            c[2] = side ? bx.n[2] - 1 : 0, c[0] = 1 + (int)(r % m[0]), c[1] = 1 + (int)(r / m[0]);
+            d = 2;
+        }
+        face_update(w, at(), kg(), Inward(bx, d, d == 0 ? c[0] : (d == 1 ? c[1] : c[2])));
+        return;
     }
+    q -= 2u * (fx + fy + fz);
+    // edges along x, y, z, the other two coordinates at 0 or n - 1 (4 combinations)
+    const int e = q < 4u * m[0] ? 0 : (q < 4u * (m[0] + m[1]) ? 1 : 2);
+    q -= e == 0 ? 0u : (e == 1 ? 4u * m[0] : 4u * (m[0] + m[1]));
+    const unsigned me = e == 0 ? m[0] : (e == 1 ? m[1] : m[2]), combo = q / me;
+    const int run = 1 + (int)(q % me);
+    const int a = e == 0 ? 1 : 0, b = e == 2 ? 1 : 2;  // the normals' axes
+    const int ca = (combo & 1u) ? (a == 0 ? bx.n[0] : bx.n[1]) - 1 : 0, cb = (combo & 2u) ? (b == 1 ? bx.n[1] : bx.n[2]) - 1 : 0;
+    c[0] = e == 0 ? run : ca;
+    c[1] = e == 1 ? run : (e == 0 ? ca : cb);
+    c[2] = e == 2 ? run : cb;
+    edge_update(w, at(), kg(), Inward(bx, a, ca), Inward(bx, b, cb));
 }
 
-// edge nodes (two wall coordinates): edges along axis a, the other two axes
-// at 0 or n - 1 (4 combinations); every edge node reads only face and
-// interior nodes, so the edges run in parallel, and the corners, which read
-// edge nodes, follow
-__host__ __device__ __forceinline__ long long edge_count(const BoxDev &bx)
+// corner t of 8
+template <class S>
+__device__ __forceinline__ void corner_update(const BoxDev &bx, unsigned t, const S &w)
 {
-    return 4LL * (bx.n[0] - 2) + 4LL * (bx.n[1] - 2) + 4LL * (bx.n[2] - 2);
-}
-__device__ __forceinline__ void edge_node(const BoxDev &bx, long long t, int c[3])
-{
-    const int n[3] = {bx.n[0], bx.n[1], bx.n[2]};
-    long long cnt[3];
-    for (int a = 0; a < 3; ++a) cnt[a] = 4LL * (n[a] - 2);
-    long long q = t;
-    int a = 0;
-    while (q >= cnt[a]) {
-        q -= cnt[a];
-        ++a;
-    }
-    const int combo = (int)(q / (n[a] - 2));
-    const int along = 1 + (int)(q % (n[a] - 2));
-    const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
-    c[a] = along;
-    c[b1] = (combo & 1) ? n[b1] - 1 : 0;
-    c[b2] = (combo & 2) ? n[b2] - 1 : 0;
-}
-__device__ __forceinline__ void corner_node(const BoxDev &bx, int t, int c[3])
-{
-    for (int d = 0; d < 3; ++d) c[d] = (t >> d) & 1 ? bx.n[d] - 1 : 0;
+    int c[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) c[d] = (t >> d) & 1u ? bx.n[d] - 1 : 0;
+    const long long i = c[0] + (long long)bx.n[0] * (c[1] + (long long)bx.n[1] * c[2]);
+    const int kg = bx.ga == 0 ? c[0] : (bx.ga == 1 ? c[1] : c[2]);
+    typename S::T tw = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) tw += along(w, i, kg, Inward(bx, d, c[d]));
+    w.store(i, kg, tw / typename S::T(3));
 }
 
-// one wall node: on the FP64 state Q (refreshing Dn and Wf when given), or,
-// with Q == nullptr, on the FP32 stage primitives Ww
-__device__ __forceinline__ void wall_node(const BoxDev &bx, const int c[3], double *Q, float *Dn, float *Wf, float *Ww)
+// the FP64 state Q (refreshing Dn and Wf when given), or, with Q == nullptr, the
+// FP32 stage primitives Ww
+__device__ __forceinline__ void wall_node(const BoxDev &bx, unsigned t, double *Q, float *Dn, float *Wf, float *Ww)
 {
     if (Q)
-        set_wall_node(bx, Q, c, Dn, Wf);
+        wall_update(bx, t, WallState{bx, Q, Dn, Wf});
     else
-        set_wall_node_w(bx, Ww, c);
+        wall_update(bx, t, WallStage{bx, Ww});
+}
+__device__ __forceinline__ void corner_node(const BoxDev &bx, unsigned t, double *Q, float *Dn, float *Wf, float *Ww)
+{
+    if (Q)
+        corner_update(bx, t, WallState{bx, Q, Dn, Wf});
+    else
+        corner_update(bx, t, WallStage{bx, Ww});
 }
 
 }  // namespace
