@@ -50,7 +50,9 @@ struct LedgerScope {
 // Device registers of a box.
 //   FP64 form: Q = Qn, Qs, acc (15 FP64 fields); W (6 FP64); R (5 FP64).
 //   Mixed form: Q = Qn (5 FP64 fields); W = slab of two FP32 primitive sets
-//     W0, W1 (12 fields); R = slab of R, K, Dn (15 FP32 fields).  Between
+//     W0, W1 of five fields each in six slots (12 in all, so that the bytes a
+//     point that memory limits are planned with stay as they are); R = slab of
+//     R, K, Dn (15 FP32 fields).  Between
 //     steps W0 and Dn hold the primitives and the base deviation of Qn, and
 //     the filter borrows both slabs as FP64 temporaries.
 //   Compact viscous terms (visc_compact): Gv, 12 fields of the stage's

@@ -172,13 +172,13 @@ struct BoxDev {
     int *err;          // device error word: set by a kernel whose bounded wait gave up
 };
 
-// Mixed form: the FP32 primitives W = (rho', u, v, w, p', H') of a state from
+// Mixed form: the FP32 primitives W = (rho', u, v, w, p') of a state from
 // its FP32 deviation from the hydrostatic base, D = (rho - rho_b, m_x, m_y,
-// m_z, E - E_b), with p' = (gamma - 1)(E' - rho |V|^2 / 2) and H' = E' + p'.
+// m_z, E - E_b), with p' = (gamma - 1)(E' - rho |V|^2 / 2).
 // Every kernel that forms the primitives of a stored state uses this one
 // function, so a state has the same FP32 primitives whichever kernel computed
 // them (a run resumed from nopcs_set_state continues bit for bit).
-__device__ __forceinline__ void prim_from_deviation(float rho_b, float gm1, const float D[5], float Wv[6])
+__device__ __forceinline__ void prim_from_deviation(float rho_b, float gm1, const float D[5], float Wv[5])
 {
     // fixed-order arithmetic (no contraction left to the compiler)
     const float ir = __fdividef(1.0f, __fadd_rn(rho_b, D[0]));
@@ -190,7 +190,6 @@ __device__ __forceinline__ void prim_from_deviation(float rho_b, float gm1, cons
     Wv[2] = v;
     Wv[3] = w;
     Wv[4] = pd;
-    Wv[5] = __fadd_rn(D[4], pd);
 }
 
 // ---- launchers (line_kernels.cu) -------------------------------------------

@@ -27,7 +27,7 @@ __device__ __forceinline__ void coords(const BoxDev &bx, long long p, int c[3])
 // with (rho_b, p_b, H_b) the hydrostatic base in the base-subtracted form and
 // zero in the plain form.  The mixed form takes the two large differences
 // rho - rho_b and E - E_b in FP64 and the rest in FP32, using
-// p - p_b = (gamma - 1)(E - E_b - rho |V|^2 / 2) and H - H_b = (E - E_b) + (p - p_b).
+// p - p_b = (gamma - 1)(E - E_b - rho |V|^2 / 2); it keeps the first five.
 // ---------------------------------------------------------------------------
 // W (and the deviation D_n, mixed form) of one point of the FP64 state
 template <typename T>
@@ -49,10 +49,10 @@ __device__ __forceinline__ void prep_point(const BoxDev &bx, long long p, int kg
         // the primitives from it exactly as the stage kernels form them
         const float D[5] = {narrow_f64(r - bx.rho_b64[kg]), narrow_f64(mx), narrow_f64(my), narrow_f64(mz),
                             narrow_f64(E - bx.E_b64[kg])};
-        float Wv[6];
+        float Wv[5];
         prim_from_deviation(bx.rho_b32[kg], (float)(bx.gamma - 1.0), D, Wv);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) W[k * np + p] = Wv[k];
+        for (int k = 0; k < 5; ++k) W[k * np + p] = Wv[k];
         if (Dn) {
 #pragma unroll
             for (int k = 0; k < 5; ++k) Dn[k * np + p] = D[k];

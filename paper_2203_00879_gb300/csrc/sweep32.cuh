@@ -18,13 +18,13 @@
 //   march_body (lines along y, z): a thread walks one line; consecutive
 //     threads take consecutive lines, so loads and stores coalesce, and no
 //     thread talks to another: no barrier anywhere.  Bound by HBM: at
-//     1024 x 512 x 512 the y and z flux sweeps take 2.67 and 2.73 ms (64 B a
-//     point, 0.95 and 0.93 of the measured copy bandwidth); the sub-domain
+//     1024 x 512 x 512 the y and z flux sweeps take 2.49 and 2.52 ms (60 B a
+//     point, 0.95 and 0.94 of the measured copy bandwidth); the sub-domain
 //     tiles with end rows and barriers took 3.56 and 3.62, held up by their
 //     alternating load, solve and store phases.
 //   scan_body (lines along x): a lane solves 8 consecutive points and takes
 //     the recurrences' state from its three neighbour lanes by shuffles.
-//     2.09 ms (44 B a point, 0.83 of the copy bandwidth; two thirds of the
+//     1.99 ms (40 B a point, 0.79 of the copy bandwidth; two thirds of the
 //     issue slots and three quarters of the shared-memory cycles used) against
 //     3.71 for whole lines in block-wide phases.
 // One field at 512^3 (8 B a point), x, y, z: 239, 240, 243 us against 469, 546,
@@ -54,9 +54,10 @@ struct Sweep32Args {
     int nch, tot;          // scan: 8-point chunks per line, chunks in all
     int kind;              // scan: 0 short lines, 1 single points, 2 four points a lane at a time
     int ga;                // gravity axis
-    const float *in[6];
+    const float *in[5];
     float *out[5];
     const float *b0, *b1, *b2;  // base tables along gravity, as LineArgs
+    float hp;              // gamma / (gamma - 1)
     float b[4];            // right-hand-side weights, normalised and scaled
     float c, g1;           // limit factor, 1 / (1 + c)
     float pw[SC_P], pw16;  // scan: (-c)^1 .. (-c)^8 and (-c)^16
@@ -72,7 +73,7 @@ template <int MODE>
 struct SweepMode {
     static constexpr bool SINGLE = MODE == MODE_FIELD || MODE == MODE_FIELD2;
     static constexpr int NF = SINGLE ? 1 : (MODE == MODE_VGRAD || MODE == MODE_VDIV ? 4 : 5);
-    static constexpr int NIN = SINGLE ? 1 : (MODE == MODE_FLUX ? 6 : (MODE == MODE_VDIV ? 4 : 5));
+    static constexpr int NIN = SINGLE ? 1 : (MODE == MODE_VDIV ? 4 : 5);
     static constexpr int REACH = sweep_reach(MODE);
     static constexpr int HW = MODE == MODE_FILTER ? 3 : 2;    // right-hand-side half-width
     static constexpr int NEXP = MODE == MODE_FILTER ? 3 : 2;  // explicit rows at a wall
@@ -92,12 +93,19 @@ __host__ __device__ constexpr bool sweep_adds(int mode, int axis)
 
 // The line quantities of one point from its inputs v and base values bb: the
 // inviscid flux along AXIS (Eqs. ge3-ge5), u, v, w, T, or the inputs
-// themselves.  Fixed-order arithmetic: the same bits in every kernel.
+// themselves.  The enthalpy H = H_b + gamma / (gamma - 1) p' + rho |V|^2 / 2 is
+// formed here from the primitives: stored, it was a sixth field for the three
+// sweeps to read and the stage kernel to write (1024 x 512 x 512: x, y, z 2.09,
+// 2.63, 2.71 ms, stage 6.98; now 1.99, 2.49, 2.52 and 6.89), and its rounding
+// is lost against that of H_b, which is thousands of times larger.  Fixed-order
+// arithmetic: the same bits in every kernel.
 template <int MODE, int AXIS>
-__device__ __forceinline__ void sweep_point(const float *v, const float *bb, float *f)
+__device__ __forceinline__ void sweep_point(const float *v, const float *bb, const float hp, float *f)
 {
     if constexpr (MODE == MODE_FLUX) {
-        const float rho = __fadd_rn(bb[0], v[0]), H = __fadd_rn(bb[1], v[5]);
+        const float rho = __fadd_rn(bb[0], v[0]);
+        const float q = __fmaf_rn(v[3], v[3], __fmaf_rn(v[2], v[2], __fmul_rn(v[1], v[1])));
+        const float H = __fadd_rn(bb[1], __fmaf_rn(hp, v[4], __fmul_rn(__fmul_rn(0.5f, rho), q)));
         const float ud = v[1 + AXIS], m = __fmul_rn(rho, ud);
         f[0] = m;
 #pragma unroll
@@ -216,9 +224,9 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
         if constexpr (NB > 0 && GROW) {
             float bb[3] = {a.b0[row], a.b1[row], 0.0f};
             if constexpr (NB > 2) bb[2] = a.b2[row];
-            sweep_point<MODE, AXIS>(v, bb, f);
+            sweep_point<MODE, AXIS>(v, bb, a.hp, f);
         } else {
-            sweep_point<MODE, AXIS>(v, bc, f);
+            sweep_point<MODE, AXIS>(v, bc, a.hp, f);
         }
     };
     auto put = [&](int slot, const float *d) {
@@ -525,7 +533,7 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
                 float u[NIN];
 #pragma unroll
                 for (int m = 0; m < NIN; ++m) u[m] = v[k][m][e];
-                sweep_point<MODE, 0>(u, bb[k][e], f[e]);
+                sweep_point<MODE, 0>(u, bb[k][e], a.hp, f[e]);
             }
             const int pos = 32 * E * (kb + k) + E * lane;
             float *const t = tile + pos + 4 * (pos >> 5);
@@ -545,7 +553,7 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
 #pragma unroll
         for (int m = 0; m < NF; ++m) f[m] = 0.0f;
         if constexpr (SHORT) {
-            if (ein) sweep_point<MODE, 0>(eu, ey, f);
+            if (ein) sweep_point<MODE, 0>(eu, ey, a.hp, f);
         }
         float *const t = tile + (lane < 4 ? lane - 4 : 288 + lane - 4);
 #pragma unroll

@@ -120,11 +120,12 @@ void sweep32_geometry(int axis, const int n[3], Sweep32Args &a)
 bool flux32_args(const LineOpDev &op, int axis, const BoxDev &bx, const float *W, float *R, Sweep32Args &a)
 {
     if (!sweep32_operator(op, sweep_reach(MODE_FLUX), -bx.inv_h[axis], a)) return false;
-    for (int k = 0; k < 6; ++k) a.in[k] = W + (size_t)k * bx.np;
+    for (int k = 0; k < 5; ++k) a.in[k] = W + (size_t)k * bx.np;
     for (int k = 0; k < 5; ++k) a.out[k] = R + (size_t)k * bx.np;
     a.ga = bx.ga;
     a.b0 = bx.rho_b32;
     a.b1 = bx.H_b32;
+    a.hp = (float)(bx.gamma / (bx.gamma - 1.0));
     sweep32_geometry(axis, bx.n, a);
     return true;
 }

@@ -34,7 +34,7 @@ struct VArgs {
     T ih2[3];             // 1 / (2 h)
     int ga, zc;           // gravity axis, planes per block
     T gm2, iRe, kq, S1, S, c0, c1, g;
-    const T *W[6];
+    const T *W[5];
     const T *rho_b, *p_b;                 // base tables (zeros in the plain form)
     const float *T_b, *ip_b, *ir_b;       // mixed form: T_b, 1/p_b, 1/rho_b
     const T *R[5];
@@ -45,7 +45,7 @@ struct VArgs {
     T *Rout[5];                           // stage 0: right-hand side out
     double *Qn[5], *acc[5], *Qout[5];     // FP64 stage registers
     float *Kacc[5], *Dn[5];               // mixed form: slope sum, deviation of Q_n
-    T *Wn[6];                             // mixed form: next stage's W
+    T *Wn[5];                             // mixed form: next stage's W
     const double *rho_b64, *E_b64;        // mixed form: base state for the deviation of Q_n
     float gm1;                            // gamma - 1
 };
@@ -390,10 +390,10 @@ __device__ __forceinline__ V4<T> flux_G(const ViscK<T> &k, const V4<T> &q, const
 // primitives of a stage state from its FP32 deviation D = (rho', m_x, m_y, m_z, E')
 __device__ __forceinline__ void prim_from_dev(const VArgs<float> &a, int p, int kg, const float D[5])
 {
-    float Wv[6];
+    float Wv[5];
     prim_from_deviation(a.rho_b[kg], a.gm1, D, Wv);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a.Wn[k][p] = Wv[k];
+    for (int k = 0; k < 5; ++k) a.Wn[k][p] = Wv[k];
 }
 
 // Mixed form of the classical RK4 stage.  The slopes are FP32 (they are FP32
@@ -714,7 +714,7 @@ VArgs<T> make_vargs(const BoxDev &bx, const T *W, const T *R, int stage, const S
     a.c0 = (T)bx.mub_coef0;
     a.c1 = (T)bx.mub_coef1;
     a.g = (T)bx.g;
-    for (int k = 0; k < 6; ++k) a.W[k] = W + (size_t)k * bx.np;
+    for (int k = 0; k < 5; ++k) a.W[k] = W + (size_t)k * bx.np;
     if constexpr (sizeof(T) == 8) {
         a.rho_b = (const T *)bx.rho_b64;
         a.p_b = (const T *)bx.p_b64;
@@ -741,7 +741,7 @@ VArgs<T> make_vargs(const BoxDev &bx, const T *W, const T *R, int stage, const S
         a.Kacc[k] = fp(g.Kacc, k);
         a.Dn[k] = fp(g.Dn, k);
     }
-    for (int k = 0; k < 6; ++k) a.Wn[k] = fp(g.Wn, k);
+    for (int k = 0; k < 5; ++k) a.Wn[k] = fp(g.Wn, k);
     a.rho_b64 = bx.rho_b64;
     a.E_b64 = bx.E_b64;
     a.gm1 = (float)(bx.gamma - 1.0);

@@ -26,8 +26,8 @@
 //
 // Bound by issue slots and latency (stage 2 at 256^3: 56% of the issue slots,
 // 568 instructions a node, 57% of the HBM cycles; 24 warps an SM, held by 80
-// registers).  Mean over the stages at 1024 x 512 x 512: 6.98 ms (138 B a
-// point, 0.78 of the measured copy bandwidth) against 8.04 with a five-plane
+// registers).  Mean over the stages at 1024 x 512 x 512: 6.89 ms (133 B a
+// point, 0.76 of the measured copy bandwidth) against 8.04 with a five-plane
 // ring, G_v in shared memory and two barriers per plane; at 256^3 0.526
 // against 0.594, at 48^3 17 us against 31.  Measured slower: two rows a thread
 // in 32 x 16 tiles (128 registers, 16 warps: 431 instructions a node, but 7.58

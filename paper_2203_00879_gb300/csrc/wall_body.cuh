@@ -63,12 +63,12 @@ struct WallState {
         Q[4 * np + i] = E;
         if (Dn) {
             const float Dv[5] = {(float)(r - bx.rho_b64[kg]), 0.0f, 0.0f, 0.0f, (float)(E - bx.E_b64[kg])};
-            float Wv[6];
+            float Wv[5];
             prim_from_deviation(bx.rho_b32[kg], (float)(bx.gamma - 1.0), Dv, Wv);
 #pragma unroll
             for (int k = 0; k < 5; ++k) Dn[k * np + i] = Dv[k];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) Wf[k * np + i] = Wv[k];
+            for (int k = 0; k < 5; ++k) Wf[k * np + i] = Wv[k];
         }
     }
 };
@@ -106,10 +106,8 @@ struct WallStage {
     {
         const long long np = bx.np;
         const float Ed = energy(W[i], kg, dT);
-        const float pd = (float)(bx.gamma - 1.0) * Ed;
         W[np + i] = W[2 * np + i] = W[3 * np + i] = 0.0f;
-        W[4 * np + i] = pd;
-        W[5 * np + i] = Ed + pd;
+        W[4 * np + i] = (float)(bx.gamma - 1.0) * Ed;
     }
 };
 
