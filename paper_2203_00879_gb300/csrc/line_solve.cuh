@@ -10,7 +10,10 @@
 //      inputs in registers and writing the forward values in place,
 //   3. back-substitutes in place,
 // leaving the derivative (or filtered value) of rows s .. e in place, times
-// osc when SCALED.
+// osc: the factor is folded into the right-hand-side weights, the end values and
+// the explicit rows, and past the tabulated factors the reciprocal pivot into the
+// weights as well, so that a row costs six multiplications and additions instead
+// of eight (FP64 runs at 1/64 of the FP32 rate: its count decides the time).
 #pragma once
 
 #include "nopcs_internal.cuh"
@@ -55,7 +58,7 @@ __device__ __forceinline__ T dot_col(const T *c, const T *f, int len, int LP)
 // org: the row at col[0]; gs / ge: the end values at rows s and e (ge unused
 // when e == s); tcp / tiv: the first KC Thomas factors (the rest equal their
 // limits cpL / invL).
-template <typename T, int MODE, bool SCALED>
+template <typename T, int MODE>
 __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, int LP, int org, T gs, T ge,
                                                    const T *tcp, const T *tiv, int KC, const int *rec, T osc)
 {
@@ -65,7 +68,8 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
     const int lene = rec[8];
     const int lo = rec[10], hi = rec[11];
     const int N = op.N;
-    auto out = [&](T v) { return SCALED ? v * osc : v; };
+    gs *= osc;
+    ge *= osc;
     // explicit wall-closure rows strictly inside the sub-domain
     T exL[NEXP], exH[NEXP];
 #pragma unroll
@@ -77,7 +81,7 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
 #pragma unroll
             for (int j = 0; j < 5; ++j)
                 if (op.ex[r][j] != 0.0) acc += (T)op.ex[r][j] * col[(size_t)(j - tlo) * LP];
-            exL[r] = acc;
+            exL[r] = osc * acc;
         }
         const int rh = N - 1 - r;
         if (rh > s && rh < e) {
@@ -85,7 +89,7 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
 #pragma unroll
             for (int j = 0; j < 5; ++j)
                 if (op.ex[r][j] != 0.0) acc += (T)op.ex[r][j] * col[(size_t)(N - 1 - j - tlo) * LP];
-            exH[r] = (T)op.ex_sign * acc;
+            exH[r] = osc * ((T)op.ex_sign * acc);
         }
     }
     // 2./3. Thomas over the implicit rows lo..hi; forward values overwrite
@@ -95,7 +99,7 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
         const T al = (T)op.alpha;
         const T gL = lo == s + 1 ? gs : exL[NEXP - 1];
         const T gR = hi == e - 1 ? ge : exH[NEXP - 1];
-        const T r0 = (T)op.rb[0], r1 = (T)op.rb[1], r2 = (T)op.rb[2], r3 = (T)op.rb[3];
+        T r0 = osc * (T)op.rb[0], r1 = osc * (T)op.rb[1], r2 = osc * (T)op.rb[2], r3 = osc * (T)op.rb[3];
         const T cL = (T)op.cpL, iL = (T)op.invL;
         T win[2 * W + 1];
         const T *pin = col + (size_t)(lo - W - tlo) * LP;
@@ -106,7 +110,7 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
         T dprev = 0;
         // one forward row: right-hand side from the window, minus the
         // coupling `adj` to a known end value, then the elimination
-        auto fwd = [&](T iv, T adj) {
+        auto right = [&] {
             win[2 * W] = *pin;
             pin += LP;
             T rhs;
@@ -116,12 +120,15 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
                 rhs = r0 * win[2] + r1 * (win[3] + win[1]) + r2 * (win[4] + win[0]);
             else
                 rhs = r0 * (win[3] - win[1]) + r1 * (win[4] - win[0]);
-            const T dp = (rhs - adj - al * dprev) * iv;
+#pragma unroll
+            for (int j = 0; j < 2 * W; ++j) win[j] = win[j + 1];
+            return rhs;
+        };
+        auto fwd = [&](T iv, T adj) {
+            const T dp = (right() - adj - al * dprev) * iv;
             *pout = dp;
             pout += LP;
             dprev = dp;
-#pragma unroll
-            for (int j = 0; j < 2 * W; ++j) win[j] = win[j + 1];
         };
         // first row carries the left end value (and the right one if m == 1)
         fwd(tiv[0], al * gL + (m == 1 ? al * gR : T(0)));
@@ -129,35 +136,46 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
         int r = 1;
 #pragma unroll 4
         for (; r < kmid; ++r) fwd(tiv[r], T(0));
+        if (r < m - 1) {
+            const T q0 = r0, q1 = r1, q2 = r2, q3 = r3;
+            r0 *= iL;
+            r1 *= iL;
+            r2 *= iL;
+            r3 *= iL;
 #pragma unroll 4
-        for (; r < m - 1; ++r) fwd(iL, T(0));
+            for (; r < m - 1; ++r) {
+                dprev = right() - cL * dprev;
+                *pout = dprev;
+                pout += LP;
+            }
+            r0 = q0, r1 = q1, r2 = q2, r3 = q3;
+        }
         if (m > 1) fwd(m - 1 < KC ? tiv[m - 1] : iL, al * gR);
         // back substitution from row hi - 1 down to lo
         T x = dprev;
-        if (SCALED) pout[-(ptrdiff_t)LP] = out(x);  // row hi
-        pout -= 2 * (size_t)LP;                      // row hi - 1
+        pout -= 2 * (size_t)LP;  // row hi - 1
         r = m - 2;
 #pragma unroll 4
         for (; r >= KC; --r) {
             x = *pout - cL * x;
-            *pout = out(x);
+            *pout = x;
             pout -= LP;
         }
 #pragma unroll 4
         for (; r >= 0; --r) {
             x = *pout - tcp[r] * x;
-            *pout = out(x);
+            *pout = x;
             pout -= LP;
         }
     }
     // explicit values into their rows
-    col[(size_t)(s - tlo) * LP] = out(gs);
-    if (lene > 0) col[(size_t)(e - tlo) * LP] = out(ge);
+    col[(size_t)(s - tlo) * LP] = gs;
+    if (lene > 0) col[(size_t)(e - tlo) * LP] = ge;
 #pragma unroll
     for (int r = 0; r < NEXP; ++r) {
-        if (r > s && r < e) col[(size_t)(r - tlo) * LP] = out(exL[r]);
+        if (r > s && r < e) col[(size_t)(r - tlo) * LP] = exL[r];
         const int rh = N - 1 - r;
-        if (rh > s && rh < e) col[(size_t)(rh - tlo) * LP] = out(exH[r]);
+        if (rh > s && rh < e) col[(size_t)(rh - tlo) * LP] = exH[r];
     }
 }
 
