@@ -43,7 +43,7 @@ constexpr int BMARCH = 128, BU = 4;
 // spreads over many blocks instead of holding the box's next phase behind a few
 // long items
 constexpr unsigned WALL_CHUNK = 4 * BT;
-enum { PH_SX = 0, PH_SY, PH_SZ, PH_VISC, PH_WALL, PH_CORNER, NPH };
+enum { PH_SX = 0, PH_SY, PH_SZ, PH_VISC, PH_WALL, NPH };
 
 struct BStage {
     Sweep32Args sw[3];
@@ -226,14 +226,14 @@ __global__ void __launch_bounds__(BT, 2) batch_step_kernel(const BParams p)
                 case PH_SY: run_march<1>(*ssw, v, reinterpret_cast<float *>(smraw)); break;
                 case PH_SZ: run_march<2>(*ssw, v, reinterpret_cast<float *>(smraw)); break;
                 case PH_VISC: run_visc_any(*sva, v % B.gx, (v / B.gx) % B.gy, v / (B.gx * B.gy), smraw); break;
-                case PH_WALL: {
-                    const unsigned t1 = min(wall_count(B.bx), (unsigned)(v + 1) * WALL_CHUNK);
-                    for (unsigned t = (unsigned)v * WALL_CHUNK + threadIdx.x; t < t1; t += BT)
+                default: {  // the walls, block 0 the corners
+                    if (v == 0) {
+                        corner_block(B.bx, threadIdx.x, S.Q, S.Dn, S.Wf, S.Ww);
+                        break;
+                    }
+                    const unsigned t1 = min(wall_count(B.bx), (unsigned)v * WALL_CHUNK);
+                    for (unsigned t = (unsigned)(v - 1) * WALL_CHUNK + threadIdx.x; t < t1; t += BT)
                         wall_node(B.bx, t, S.Q, S.Dn, S.Wf, S.Ww);
-                    break;
-                }
-                default: {  // the corners, which read the edges
-                    if (threadIdx.x < 8) corner_node(B.bx, threadIdx.x, S.Q, S.Dn, S.Wf, S.Ww);
                 }
                 }
                 __syncthreads();  // the next block of the item reuses the shared memory
@@ -308,8 +308,7 @@ cudaError_t batch_plan_build(const std::vector<BatchBoxIn> &in, BatchPlan **out,
                 S.Ww = nullptr;
             }
         }
-        B.ntile[PH_WALL] = (int)((wall_count(I.bx) + WALL_CHUNK - 1) / WALL_CHUNK);
-        B.ntile[PH_CORNER] = 1;
+        B.ntile[PH_WALL] = 1 + (int)((wall_count(I.bx) + WALL_CHUNK - 1) / WALL_CHUNK);
         // blocks per item: about a quarter of a GPU wave per phase of a big
         // box, single blocks for small ones
         for (int ph = 0; ph < NPH; ++ph) {

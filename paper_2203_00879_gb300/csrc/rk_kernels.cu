@@ -103,14 +103,13 @@ __global__ void filter_update_kernel(const BoxDev bx, double *__restrict__ Q, co
 
 __global__ void wall_kernel(const BoxDev bx, double *Q, float *Dn, float *Wf, float *Ww)
 {
+    if (blockIdx.x == 0) {
+        corner_block(bx, threadIdx.x, Q, Dn, Wf, Ww);
+        return;
+    }
     const unsigned tot = wall_count(bx);
-    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += gridDim.x * blockDim.x)
+    for (unsigned t = (blockIdx.x - 1) * blockDim.x + threadIdx.x; t < tot; t += (gridDim.x - 1) * blockDim.x)
         wall_node(bx, t, Q, Dn, Wf, Ww);
-}
-
-__global__ void wall_corner_kernel(const BoxDev bx, double *Q, float *Dn, float *Wf, float *Ww)
-{
-    if (threadIdx.x < 8) corner_node(bx, threadIdx.x, Q, Dn, Wf, Ww);
 }
 
 // ---------------------------------------------------------------------------
@@ -361,10 +360,7 @@ cudaError_t launch_filter_update(const BoxDev &bx, double *Q, const float *Fd, f
 
 cudaError_t launch_wall_bc(const BoxDev &bx, double *Q, float *Dn, float *Wf, float *Ww, cudaStream_t st)
 {
-    wall_kernel<<<grid_for(wall_count(bx), 128), 128, 0, st>>>(bx, Q, Dn, Wf, Ww);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    wall_corner_kernel<<<1, 32, 0, st>>>(bx, Q, Dn, Wf, Ww);
+    wall_kernel<<<1 + grid_for(wall_count(bx), 128), 128, 0, st>>>(bx, Q, Dn, Wf, Ww);
     return cudaGetLastError();
 }
 

@@ -19,11 +19,15 @@ namespace {
 // Faces and edges are set in one pass: an edge node works out the four face
 // temperatures it needs from the four interior nodes behind them instead of
 // waiting for them, so nothing reads what another thread writes (the density of
-// a wall node is not written).  The corners follow, from the stored edges.
+// a wall node is not written).  A corner reads the two nodes next to it on each
+// of its edges, so one block sets the 48 such edge nodes of a box and then, after
+// a barrier, its corners.
 // Bound by latency at all but the largest sizes: every load of a node is issued
-// before its first use.  Faces, edges and corners as three launches with
-// branches between the loads: 31 us per stage in boxes of 32 to 128 points, now
-// 22; 256^3 70 us, now 57.
+// before its first use, and a stage has one launch.  Between two events on the
+// stream at 48^3 and 256^3: 28 and 70 us as three launches (faces, edges,
+// corners) with branches between the loads, 20 and 57 with the faces and edges
+// in one, now 14 at 48^3.  (Edges and corners recursing to the interior, nothing
+// shared: 50 us at 48^3.)
 // ---------------------------------------------------------------------------
 
 // On the FP64 state (refreshing D_n and W when given).  A value is a
@@ -156,6 +160,20 @@ __device__ __forceinline__ void edge_update(const S &w, long long i, int kg, con
                     w.extrapolate(kg, kg + b.k, fb[0], kg + 2 * b.k, fb[1])) / T(2));
 }
 
+// node `run` of edge e = 4 x its axis + the sides of the other two coordinates
+template <class S>
+__device__ __forceinline__ void edge_node(const BoxDev &bx, unsigned e, int run, const S &w)
+{
+    const int ax = (int)(e >> 2), a = ax == 0 ? 1 : 0, b = ax == 2 ? 1 : 2;  // a, b: the normals' axes
+    const int ca = (e & 1u) ? (a == 0 ? bx.n[0] : bx.n[1]) - 1 : 0, cb = (e & 2u) ? (b == 1 ? bx.n[1] : bx.n[2]) - 1 : 0;
+    int c[3];
+    c[0] = ax == 0 ? run : ca;
+    c[1] = ax == 1 ? run : (ax == 0 ? ca : cb);
+    c[2] = ax == 2 ? run : cb;
+    const long long i = c[0] + (long long)bx.n[0] * (c[1] + (long long)bx.n[1] * c[2]);
+    edge_update(w, i, bx.ga == 0 ? c[0] : (bx.ga == 1 ? c[1] : c[2]), Inward(bx, a, ca), Inward(bx, b, cb));
+}
+
 // Wall nodes in order: faces (one wall coordinate), edges (two).
 // A box of fewer than 2^31 points has fewer than 2^31 of them.
 __host__ __device__ __forceinline__ unsigned face_count(const BoxDev &bx)
@@ -172,7 +190,8 @@ __host__ __device__ __forceinline__ unsigned wall_count(const BoxDev &bx)
 {
     return face_count(bx) + edge_count(bx);
 }
-// wall node t (a face or an edge node) of the state seen through w
+// wall node t (a face or an edge node) of the state seen through w; the edge
+// nodes that a corner reads are left to corner_block
 template <class S>
 __device__ __forceinline__ void wall_update(const BoxDev &bx, unsigned q, const S &w)
 {
@@ -205,13 +224,8 @@ __device__ __forceinline__ void wall_update(const BoxDev &bx, unsigned q, const 
     const int e = q < 4u * m[0] ? 0 : (q < 4u * (m[0] + m[1]) ? 1 : 2);
     q -= e == 0 ? 0u : (e == 1 ? 4u * m[0] : 4u * (m[0] + m[1]));
     const unsigned me = e == 0 ? m[0] : (e == 1 ? m[1] : m[2]), combo = q / me;
-    const int run = 1 + (int)(q % me);
-    const int a = e == 0 ? 1 : 0, b = e == 2 ? 1 : 2;  // the normals' axes
-    const int ca = (combo & 1u) ? (a == 0 ? bx.n[0] : bx.n[1]) - 1 : 0, cb = (combo & 2u) ? (b == 1 ? bx.n[1] : bx.n[2]) - 1 : 0;
-    c[0] = e == 0 ? run : ca;
-    c[1] = e == 1 ? run : (e == 0 ? ca : cb);
-    c[2] = e == 2 ? run : cb;
-    edge_update(w, at(), kg(), Inward(bx, a, ca), Inward(bx, b, cb));
+    const int run = 1 + (int)(q % me), last = (int)me;
+    if (run > 2 && run < last - 1) edge_node(bx, 4u * (unsigned)e + combo, run, w);
 }
 
 // corner t of 8
@@ -238,12 +252,26 @@ __device__ __forceinline__ void wall_node(const BoxDev &bx, unsigned t, double *
     else
         wall_update(bx, t, WallStage{bx, Ww});
 }
-__device__ __forceinline__ void corner_node(const BoxDev &bx, unsigned t, double *Q, float *Dn, float *Wf, float *Ww)
+// The corners and the edge nodes next to them, by all threads of one block (48
+// at least).
+template <class S>
+__device__ __forceinline__ void corner_block_of(const BoxDev &bx, unsigned t, const S &w)
+{
+    if (t < 48) {
+        const unsigned e = t >> 2, k = t & 3;
+        const int last = (e < 4 ? bx.n[0] : (e < 8 ? bx.n[1] : bx.n[2])) - 2;  // of the edge's nodes 1 .. last
+        const int run = k < 2 ? 1 + (int)k : last - (int)k + 2;
+        if (k < 2 || run > 2) edge_node(bx, e, run, w);  // each node once
+    }
+    __syncthreads();
+    if (t < 8) corner_update(bx, t, w);
+}
+__device__ __forceinline__ void corner_block(const BoxDev &bx, unsigned t, double *Q, float *Dn, float *Wf, float *Ww)
 {
     if (Q)
-        corner_update(bx, t, WallState{bx, Q, Dn, Wf});
+        corner_block_of(bx, t, WallState{bx, Q, Dn, Wf});
     else
-        corner_update(bx, t, WallStage{bx, Ww});
+        corner_block_of(bx, t, WallStage{bx, Ww});
 }
 
 }  // namespace
