@@ -30,12 +30,12 @@ UNIT = "point-stage updates/s"
 # algorithmic bytes per grid point of one launch of each kernel kind
 # (mixed form; see the design notes for the derivation)
 ALG_BYTES_MIXED = {
-    "prep": 40 + 24,                   # read Q (5 f64), write W (6 f32)
-    "sweep_x": 24 + 20,                # read W, write R (5 f32)
-    "sweep_y": 24 + 40,                # read W, read+write R
-    "sweep_z": 24 + 40,
+    "prep": 40 + 20 + 20,              # read Q (5 f64), write W and the deviation (5 f32 each)
+    "sweep_x": 20 + 20,                # read W, write R (5 f32)
+    "sweep_y": 20 + 40,                # read W, read+write R
+    "sweep_z": 20 + 40,
     # stage average of W + R + Dn (+ K) in, K + W' out; stage 4 also Q_n in/out and Dn out
-    "visc_rk_update": (108 + 128 + 128 + 188) / 4.0,
+    "visc_rk_update": (104 + 124 + 124 + 180) / 4.0,
     "filter": 3 * 80,                  # three sweeps, each read+write Q
     # compact viscous terms (visc_compact): per launch of each kind
     "visc_grad": 20 + 16,              # read rho', u, v, w, p'; write 4 gradients
@@ -43,7 +43,7 @@ ALG_BYTES_MIXED = {
     "visc_div": 16 + 32,               # read 4 fluxes; reduction adds into R[1..4] (read + write)
     # visc_rk_update without the viscous terms: W0 and the velocity along gravity
     # instead of the five primitives the viscous stencils need
-    "source_rk_update": (92 + 112 + 112 + 172) / 4.0,
+    "source_rk_update": (88 + 108 + 108 + 164) / 4.0,
 }
 ALG_BYTES_FP64 = {
     "prep": 40 + 48, "sweep_x": 48 + 40, "sweep_y": 48 + 80, "sweep_z": 48 + 80,

@@ -32,18 +32,13 @@ struct LineArgs {
 
 // One block of the sub-domain sweep: block `vblock` of the launch grid
 // (sub-domain vblock % nsub of line tile vblock / nsub), in the block's
-// dynamic shared memory, threads 0 .. NT-1 working (a larger block's other
-// threads only take part in the barriers, so the arithmetic, and its
-// rounding, is that of an NT-thread launch).  The shared array is declared
-// here rather than passed in.
-template <typename T, int MODE, int AXIS, bool ALL = false>
-__device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T> &a, const unsigned vblock,
-                                          const int nt_req)
+// dynamic shared memory.  The shared array is declared here rather than passed
+// in.
+template <typename T, int MODE, int AXIS>
+__device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T> &a, const unsigned vblock)
 {
     extern __shared__ __align__(32) unsigned char smraw[];
-    // ALL: every thread of the block works (the stand-alone launch)
-    const int NT = ALL ? (int)blockDim.x : nt_req;
-    const bool worker = ALL || (int)threadIdx.x < NT;
+    const int NT = (int)blockDim.x;
     constexpr bool SINGLE = MODE == MODE_FIELD || MODE == MODE_FIELD2;  // one field in, one out
     constexpr bool VISC = MODE == MODE_VGRAD || MODE == MODE_VDIV;      // four fields out
     constexpr int NF = SINGLE ? 1 : (VISC ? 4 : 5);
@@ -101,11 +96,11 @@ __device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T>
     const T *coef = coef_ptr<T>(op);
     {
         if (!STREAM) {
-            for (int k = worker ? threadIdx.x : lens; k < lens; k += NT) cs[k] = coef[rec[6] + k];
-            for (int k = worker ? threadIdx.x : lene; k < lene; k += NT) ce[k] = coef[rec[9] + k];
+            for (int k = threadIdx.x; k < lens; k += NT) cs[k] = coef[rec[6] + k];
+            for (int k = threadIdx.x; k < lene; k += NT) ce[k] = coef[rec[9] + k];
         }
         const T *cpp = cp_ptr<T>(op), *ivp = inv_ptr<T>(op);
-        for (int k = worker ? threadIdx.x : KC; k < KC; k += NT) {
+        for (int k = threadIdx.x; k < KC; k += NT) {
             tcp[k] = cpp[k];
             tiv[k] = ivp[k];
         }
@@ -123,7 +118,7 @@ __device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T>
         if (AXIS == 0) {
             r0 = threadIdx.x & 31;
             rstep = 32;
-            l0 = worker ? (int)threadIdx.x >> 5 : nl;
+            l0 = (int)threadIdx.x >> 5;
             lstep = NT >> 5;
         } else {
             l0 = threadIdx.x % LINES;
@@ -280,10 +275,10 @@ __device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T>
         if (AXIS == 0) {
             r0 = threadIdx.x & 31;
             rstep = 32;
-            l0 = worker ? (int)threadIdx.x >> 5 : nl;
+            l0 = (int)threadIdx.x >> 5;
             lstep = NT >> 5;
         } else {
-            l0 = worker ? (int)threadIdx.x % LINES : nl;
+            l0 = (int)threadIdx.x % LINES;
             lstep = LINES;
             r0 = threadIdx.x / LINES;
             rstep = NT / LINES;
@@ -378,20 +373,18 @@ __device__ __forceinline__ void xline_flux_point(const LineArgs<T> &a, T *d, con
     d[4 * FS] = H * uu;
 }
 
-template <typename T, int MODE>
+template <typename T>
 __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const LineArgs<T> &a, T *sm,
                                                   const T *ctab, const T *tcp, const T *tiv, const int line0,
                                                   const int nl);
 
 // One block of the whole-line x sweep: lines vblock * LINES .. + LINES - 1,
 // in the block's dynamic shared memory.
-template <typename T, int MODE>
+template <typename T>
 __device__ __forceinline__ void xline_body(const LineOpDev &op, const LineArgs<T> &a, const int vblock)
 {
     extern __shared__ __align__(32) unsigned char smraw[];
-    constexpr bool SINGLE = MODE == MODE_FIELD;
-    constexpr int NF = SINGLE ? 1 : 5;
-    constexpr int NIN = SINGLE ? 1 : 6;
+    constexpr int NF = 5, NIN = 6;
     constexpr int U = 4;     // staged points in flight per thread and field
     const int N = op.N;      // = nx
     const int nx = a.n[0], ny = a.n[1];
@@ -432,29 +425,24 @@ __device__ __forceinline__ void xline_body(const LineOpDev &op, const LineArgs<T
                 const int g = g0 + u * (int)blockDim.x;
                 if (g >= N) continue;
                 T *d = sm + (size_t)l * LS + xrow(g);
-                if constexpr (SINGLE) {
-                    d[0] = v[u][0];
-                } else {
-                    xline_flux_point(a, d, FS, v[u], a.ga == 0 ? g : gl);
-                }
+                xline_flux_point(a, d, FS, v[u], a.ga == 0 ? g : gl);
             }
         }
     }
     __syncthreads();
-    xline_solve_store<T, MODE>(op, a, sm, ctab, tcp, tiv, line0, nl);
+    xline_solve_store<T>(op, a, sm, ctab, tcp, tiv, line0, nl);
 }
 
 // The solve and the store of the whole-line x sweep, once lines line0 ..
 // line0 + nl - 1 are staged in the tile sm (and a barrier has passed): the
 // columns, thread c solving sub-domain c % nsub of line (c / nsub) % nl, field
 // c / (nsub nl), in phases A-C, then the rows scaled by 1/h into the outputs.
-template <typename T, int MODE>
+template <typename T>
 __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const LineArgs<T> &a, T *sm,
                                                   const T *ctab, const T *tcp, const T *tiv, const int line0,
                                                   const int nl)
 {
-    constexpr bool SINGLE = MODE == MODE_FIELD;
-    constexpr int NF = SINGLE ? 1 : 5;
+    constexpr int NF = 5;
     constexpr int NEXP = 2;  // explicit rows at each wall (derivative)
     const int N = op.N;      // = nx
     const int nx = a.n[0];
@@ -577,17 +565,13 @@ __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const Lin
         for (int g = threadIdx.x; g < N; g += blockDim.x) {
             const int o = base + g;
             const int q = xrow(g);
-            if constexpr (SINGLE) {
-                a.out[0][o] = src[q] * a.scale;
-            } else {
 #pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    const T v = -src[(size_t)k * FS + q] * a.scale;
-                    if (a.first)
-                        a.out[k][o] = v;
-                    else
-                        atomicAdd(&a.out[k][o], v);
-                }
+            for (int k = 0; k < 5; ++k) {
+                const T v = -src[(size_t)k * FS + q] * a.scale;
+                if (a.first)
+                    a.out[k][o] = v;
+                else
+                    atomicAdd(&a.out[k][o], v);
             }
         }
     }
@@ -603,9 +587,7 @@ constexpr size_t SMEM_BUDGET = 200 * 1024;
 // single field the sub-domain tiles stay faster (0.46 ms at 512^3 against 0.50
 // with four lines and 1.42 with one), so FIELD keeps them.
 constexpr size_t XLINE_SMEM = 100 * 1024, XLINE_SMEM_MULTI = 48 * 1024;
-#ifndef XLINE_MAX_LINES
-#define XLINE_MAX_LINES 1
-#endif
+constexpr int XLINE_MAX_LINES = 1;  // up to 4 (LineOpDev::xpitch)
 
 inline int pick_lines(int pref, int rw, int nf, size_t esz)
 {
@@ -621,13 +603,11 @@ struct LineGrid {
     bool xline = false;  // the whole-line x kernel runs
 };
 
-// Geometry of one sweep along AXIS: fills a.lines, a.ntile_a, a.rt, a.rw.
-// threads_req > 0 fixes the block size (the batched kernel's); max_xlines
-// bounds the lines per block of the whole-line x kernel (FLUX along x only),
-// which needs one thread per (line, field, sub-domain) column.  False if no
-// configuration fits.
+// Geometry of one sweep along AXIS: fills a.lines, a.ntile_a, a.rt, a.rw.  The
+// whole-line x kernel (FLUX along x only) needs one thread per (line, field,
+// sub-domain) column.  False if no configuration fits.
 template <typename T, int MODE, int AXIS>
-bool line_grid(const LineOpDev &op, LineArgs<T> &a, int pref_lines, int threads_req, int max_xlines, LineGrid &g)
+bool line_grid(const LineOpDev &op, LineArgs<T> &a, int pref_lines, LineGrid &g)
 {
     constexpr bool SINGLE = MODE == MODE_FIELD || MODE == MODE_FIELD2;
     constexpr int NF = SINGLE ? 1 : (MODE == MODE_VGRAD || MODE == MODE_VDIV ? 4 : 5);
@@ -637,18 +617,17 @@ bool line_grid(const LineOpDev &op, LineArgs<T> &a, int pref_lines, int threads_
     // to keep a block busy in its solve: at 256^3 (20 columns) it was 1.7 times
     // slower than the sub-domain tiles, at 1024^3 (80 columns) 6% faster
     if (AXIS == 0 && MODE == MODE_FLUX && op.nsub * NF >= 64) {
-        for (int L = max_xlines < 4 ? max_xlines : 4; L >= 1; --L) {
-            const int pitch = op.xpitch[1][L - 1];
+        for (int L = XLINE_MAX_LINES; L >= 1; --L) {
+            const int pitch = op.xpitch[L - 1];
             const size_t bytes = ((size_t)NF * L * pitch + (size_t)op.ncoef + 2 * (size_t)kc) * sizeof(T);
             const int cols = op.nsub * NF * L;
-            const int cap = threads_req > 0 ? threads_req : 1024;
-            if (bytes > XLINE_SMEM || cols > cap) continue;
+            if (bytes > XLINE_SMEM || cols > 1024) continue;
             if (L > 1 && bytes > XLINE_SMEM_MULTI) continue;
             a.lines = L;
             a.rt = pitch;
             int threads = (cols + 31) / 32 * 32;
             if (threads < 128) threads = 128;
-            g.threads = threads_req > 0 ? threads_req : threads;
+            g.threads = threads;
             g.smem = bytes;
             g.xline = true;
             g.nblk = ((long long)a.n[1] * a.n[2] + L - 1) / L;
@@ -659,8 +638,6 @@ bool line_grid(const LineOpDev &op, LineArgs<T> &a, int pref_lines, int threads_
     a.rw = op.max_win;
     const int rows = (AXIS != 0 || !SINGLE) ? a.rw : a.rt;
     a.lines = pick_lines(pref_lines, rows, NF, sizeof(T));
-    if (threads_req > 0)
-        while (a.lines > 1 && a.lines * NF > threads_req) a.lines /= 2;
     const int Na = AXIS == 0 ? a.n[1] : a.n[0];
     const int Nc = AXIS == 2 ? a.n[1] : a.n[2];
     a.ntile_a = (Na + a.lines - 1) / a.lines;
@@ -676,7 +653,6 @@ bool line_grid(const LineOpDev &op, LineArgs<T> &a, int pref_lines, int threads_
     if (threads < 128) threads = 128;
     if (threads > 1024) threads = (a.lines * NF + 31) / 32 * 32;
     if (threads > 1024) return false;
-    if (threads_req > 0) threads = threads_req;
     const int rg = (AXIS != 0 || !SINGLE) ? (AXIS == 0 ? 1 : threads / a.lines) : 0;
     g.threads = threads;
     g.smem = ((size_t)NF * rows * (a.lines + 1) + 2 * (size_t)op.max_taps + 2 * (size_t)kc +

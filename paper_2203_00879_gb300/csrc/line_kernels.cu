@@ -31,7 +31,7 @@ namespace nopcs {
 template <typename T, int MODE, int AXIS>
 __global__ void line_kernel(const LineOpDev op, const LineArgs<T> a)
 {
-    line_body<T, MODE, AXIS, true>(op, a, blockIdx.x, 0);
+    line_body<T, MODE, AXIS>(op, a, blockIdx.x);
 }
 
 namespace {
@@ -40,7 +40,7 @@ template <typename T, int MODE, int AXIS>
 cudaError_t launch_axis(const LineOpDev &op, LineArgs<T> a, int pref_lines, cudaStream_t st)
 {
     LineGrid g;
-    if (!line_grid<T, MODE, AXIS>(op, a, pref_lines, 0, XLINE_MAX_LINES, g)) return cudaErrorInvalidConfiguration;
+    if (!line_grid<T, MODE, AXIS>(op, a, pref_lines, g)) return cudaErrorInvalidConfiguration;
     if (g.nblk <= 0) return cudaSuccess;
     if constexpr (AXIS == 0 && MODE == MODE_FLUX) {
         if (g.xline) return launch_xline_flux<T>(op, a, g.nblk, g.threads, g.smem, st);

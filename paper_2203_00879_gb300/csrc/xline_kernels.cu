@@ -9,7 +9,7 @@ namespace {
 template <typename T>
 __global__ void xline_kernel(const LineOpDev op, const LineArgs<T> a)
 {
-    xline_body<T, MODE_FLUX>(op, a, (int)blockIdx.x);
+    xline_body<T>(op, a, (int)blockIdx.x);
 }
 
 }  // namespace
