@@ -580,12 +580,8 @@ __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const Lin
 
 // ---- launch geometry (host) ----------------------------------------------------
 constexpr size_t SMEM_BUDGET = 200 * 1024;
-// whole-line x sweep: at most this much shared memory per block, and several
-// lines per block only while a block stays below the second figure.  One line
-// per block measured fastest for the five-field flux sweep at 1024^3 (14.73 ms
-// against 16.02 with two lines and 15.62 for the sub-domain tiles); for a
-// single field the sub-domain tiles stay faster (0.46 ms at 512^3 against 0.50
-// with four lines and 1.42 with one), so FIELD keeps them.
+// whole-line x flux sweep: at most this much shared memory per block, and
+// several lines per block only while a block stays below the second figure
 constexpr size_t XLINE_SMEM = 100 * 1024, XLINE_SMEM_MULTI = 48 * 1024;
 constexpr int XLINE_MAX_LINES = 1;  // up to 4 (LineOpDev::xpitch)
 
@@ -613,10 +609,21 @@ bool line_grid(const LineOpDev &op, LineArgs<T> &a, int pref_lines, LineGrid &g)
     constexpr int NF = SINGLE ? 1 : (MODE == MODE_VGRAD || MODE == MODE_VDIV ? 4 : 5);
     const int kc = sizeof(T) == 8 ? op.kconv64 : op.kconv32;
     g = LineGrid();
-    // the whole-line kernel needs enough (field, sub-domain) columns per line
-    // to keep a block busy in its solve: at 256^3 (20 columns) it was 1.7 times
-    // slower than the sub-domain tiles, at 1024^3 (80 columns) 6% faster
-    if (AXIS == 0 && MODE == MODE_FLUX && op.nsub * NF >= 64) {
+    // The whole-line kernel saves the tiles' second reading of end rows, but a
+    // warp of its solve costs the same however many of its lanes have a (field,
+    // sub-domain) column.  Nx x 96 x 96, ms, tiles and whole lines; columns of
+    // the lanes of their warps:
+    //   sub-domains of 64: Nx = 512  0.738 0.859 (40 of 64), 768  1.096 1.008 (60 of 64),
+    //     832 1.180 1.334 (65 of 96), 1024  1.440 1.551 (80 of 96), 1536  2.143 2.091 (120 of 128)
+    //   of 32: 256  0.520 0.539 (40 of 64), 512  1.019 0.948 (80 of 96), 1024  2.022 1.703 (160 of 160)
+    //   of 128: 1024  1.310 1.555 (40 of 64)
+    // so whole lines where nine lanes in ten work, or four in five with short
+    // sub-domains, whose tiles read the most rows twice; not with long ones, nor
+    // with fewer than 50 columns (none measured faster).
+    const int columns = op.nsub * NF, lanes = (columns + 31) / 32 * 32;
+    const bool filled = op.N < 48 * op.nsub ? 5 * columns >= 4 * lanes
+                                            : op.N < 96 * op.nsub && 10 * columns >= 9 * lanes;
+    if (AXIS == 0 && MODE == MODE_FLUX && columns >= 50 && filled) {
         for (int L = XLINE_MAX_LINES; L >= 1; --L) {
             const int pitch = op.xpitch[L - 1];
             const size_t bytes = ((size_t)NF * L * pitch + (size_t)op.ncoef + 2 * (size_t)kc) * sizeof(T);

@@ -20,9 +20,11 @@
 // tile and takes the end values from it.)
 //
 // Modes: FIELD / FIELD2 one field; FLUX the five inviscid fluxes along the
-// axis from the stage primitives, into R (FP64; FP32 in sweep32.cuh); FILTER five state fields; VGRAD and
+// axis from the stage primitives, into R; FILTER five state fields; VGRAD and
 // VDIV the compact viscous terms -- the derivatives of u, v, w, T, and those
-// of the four viscous-flux components along the axis, added into R[1..4].
+// of the four viscous-flux components along the axis, added into R[1..4].  All
+// in FP64; the FP32 ones are in sweep32.cuh, but for a filter whose
+// coefficient its recurrences do not take.
 #include "line_body.cuh"
 #include "sweep32.cuh"
 
