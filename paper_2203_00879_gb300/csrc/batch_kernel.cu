@@ -37,7 +37,8 @@ constexpr int BT = 256;             // threads per block (the viscous tile's)
 // and rows of theirs in flight, at two blocks per SM: a step of the 64-box
 // workload takes 39.4 ms, of one 256^3 box 9.1 ms; with 160 lines 39.4 and 9.8,
 // with 160 lines and 8 rows 42.2 and 10.7, at three blocks per SM (80 registers
-// a thread, the sweeps spill) with 96 lines and 2 rows 46.5 and 11.6.
+// a thread, the sweeps spill) with 96 lines and 2 rows 46.5 and 11.6.  (All
+// before the stage and wall kernels were changed: now 36.2 and 8.5.)
 constexpr int BMARCH = 128, BU = 4;
 // wall nodes per tile: four passes of a block, so that a box's wall phase
 // spreads over many blocks instead of holding the box's next phase behind a few

@@ -26,7 +26,7 @@ namespace {
 // before its first use, and a stage has one launch.  Between two events on the
 // stream at 48^3 and 256^3: 28 and 70 us as three launches (faces, edges,
 // corners) with branches between the loads, 20 and 57 with the faces and edges
-// in one, now 14 at 48^3.  (Edges and corners recursing to the interior, nothing
+// in one, now 14 and 45.  (Edges and corners recursing to the interior, nothing
 // shared: 50 us at 48^3.)
 // ---------------------------------------------------------------------------
 
