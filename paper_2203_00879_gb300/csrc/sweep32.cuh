@@ -570,10 +570,13 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
     const int hj = N - 1 - g0;
     const bool lo = ok && ch == 0, hi = ok && hj - (NEXP - 1) < P;
     const bool anylo = __any_sync(ALL, lo), anyhi = __any_sync(ALL, hi);
-    // weights of the three neighbours' end values in the state that enters the
-    // lane from the left and from the right; none across a line's end or from
-    // outside the warp
-    float wl[3], wr[3], kf = 0.0f;
+    // neighbours on the lane's left and right that hold chunks of its own line.
+    // Values of the others are left out by selection: a weight of zero would
+    // let a NaN or an infinity of one line through to the next.
+    const int left = ok ? min(ch, lane) : 0, right = ok ? min(a.nch - 1 - ch, 31 - lane) : 0;
+    // weights of the second and third neighbours' end values in the state that
+    // enters the lane (the first one's is 1)
+    float wl1 = a.pw[P - 1], wl2 = a.pw16, wr1 = a.pw[P - 1], wr2 = a.pw16;
     // SHORT: factor of a row, its pivot's ratio to the limit (0 for explicit
     // rows), weight at a row of the state entering from the left and right
     float cp[P], rt[P], pf[P], ps[P];
@@ -587,24 +590,11 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
         }
 #pragma unroll
         for (int j = P - 1; j >= 0; --j) ps[j] = j < P - 1 ? __fmul_rn(-cp[j], ps[j < P - 1 ? j + 1 : j]) : -cp[j];
-        const float l1 = __shfl_up_sync(ALL, pf[P - 1], 1), l2 = __shfl_up_sync(ALL, pf[P - 1], 2);
-        const float r1 = __shfl_down_sync(ALL, ps[0], 1), r2 = __shfl_down_sync(ALL, ps[0], 2);
-        wl[0] = lane > 0 ? 1.0f : 0.0f;
-        wl[1] = lane > 1 ? l1 : 0.0f;
-        wl[2] = lane > 2 ? l1 * l2 : 0.0f;
-        wr[0] = lane < 31 ? 1.0f : 0.0f;
-        wr[1] = lane < 30 ? r1 : 0.0f;
-        wr[2] = lane < 29 ? r1 * r2 : 0.0f;
-    } else {
-        const int left = ok ? min(ch, lane) : 0, right = ok ? min(a.nch - 1 - ch, 31 - lane) : 0;
-        wl[0] = left > 0 ? 1.0f : 0.0f;
-        wl[1] = left > 1 ? a.pw[P - 1] : 0.0f;
-        wl[2] = left > 2 ? a.pw16 : 0.0f;
-        wr[0] = right > 0 ? 1.0f : 0.0f;
-        wr[1] = right > 1 ? a.pw[P - 1] : 0.0f;
-        wr[2] = right > 2 ? a.pw16 : 0.0f;
-        if (ok && ch <= SC_H) kf = a.kf[ch];
+        wl1 = __shfl_up_sync(ALL, pf[P - 1], 1), wl2 = wl1 * __shfl_up_sync(ALL, pf[P - 1], 2);
+        wr1 = __shfl_down_sync(ALL, ps[0], 1), wr2 = wr1 * __shfl_down_sync(ALL, ps[0], 2);
     }
+    const bool near_lo = ok && ch <= SC_H;  // chunks that the low wall's first factors reach
+    const float kf = near_lo ? a.kf[ch] : 0.0f;
 #pragma unroll 1
     for (int m = 0; m < NF; ++m) {
         float *const t = tile + m * SC_FS;
@@ -622,7 +612,8 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
 #pragma unroll
         for (int j = 0; j < P; ++j) {
             d[j] = sweep_rhs<MODE>(a, w + 4 + j - HW, 1);
-            if constexpr (SHORT) d[j] = __fmul_rn(rt[j], d[j]);
+            // rows beyond the line's end have the next line's points in their stencils
+            if constexpr (SHORT) d[j] = j < cnt ? __fmul_rn(rt[j], d[j]) : 0.0f;
         }
         if (anylo) {
 #pragma unroll
@@ -671,7 +662,9 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
         {
             const float d1 = __shfl_up_sync(ALL, d[P - 1], 1), d2 = __shfl_up_sync(ALL, d[P - 1], 2),
                         d3 = __shfl_up_sync(ALL, SHORT ? d[P - 1] : dq, 3);
-            const float y = __fmaf_rn(wl[2], d3, __fmaf_rn(wl[1], d2, __fmul_rn(wl[0], d1)));
+            float y = left > 0 ? d1 : 0.0f;
+            if (left > 1) y = __fmaf_rn(wl1, d2, y);
+            if (left > 2) y = __fmaf_rn(wl2, d3, y);
 #pragma unroll
             for (int j = 0; j < P; ++j) d[j] = __fmaf_rn(SHORT ? pf[j] : a.pw[j], y, d[j]);
         }
@@ -693,13 +686,16 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
         {
             const float x1 = __shfl_down_sync(ALL, d[0], 1), x2 = __shfl_down_sync(ALL, d[0], 2),
                         x3 = __shfl_down_sync(ALL, SHORT ? d[0] : xq, 3);
-            const float z = __fmaf_rn(wr[2], x3, __fmaf_rn(wr[1], x2, __fmul_rn(wr[0], x1)));
+            float z = right > 0 ? x1 : 0.0f;
+            if (right > 1) z = __fmaf_rn(wr1, x2, z);
+            if (right > 2) z = __fmaf_rn(wr2, x3, z);
 #pragma unroll
             for (int j = 0; j < P; ++j) d[j] = __fmaf_rn(SHORT ? ps[j] : a.pw[P - 1 - j], z, d[j]);
         }
         if constexpr (!SHORT) {
             if (anylo) {
-                const float y = __fmul_rn(kf, __shfl_sync(ALL, d[NEXP], max(lane - ch, 0)));
+                const float x0 = __shfl_sync(ALL, d[NEXP], max(lane - ch, 0));
+                const float y = near_lo ? __fmul_rn(kf, x0) : 0.0f;
 #pragma unroll
                 for (int j = 0; j < P; ++j) d[j] = __fmaf_rn(a.pw[j], y, d[j]);
                 if (lo) {
