@@ -399,8 +399,10 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
                     float d[NF];
                     get(sb + u, d);
                     const float cp = a.cp[low ? min(ib + u, SW_TAB - 1) : SW_TAB - 1];
+                    // an explicit row (factor 0) has its own value whatever the
+                    // rows above it hold
 #pragma unroll
-                    for (int k = 0; k < NF; ++k) X[k] = __fmaf_rn(-cp, X[k], d[k]);
+                    for (int k = 0; k < NF; ++k) X[k] = cp == 0.0f ? d[k] : __fmaf_rn(-cp, X[k], d[k]);
                     if (out && ib + u < emax) emit(ib + u, X);
                 }
             }
@@ -692,7 +694,16 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
 #pragma unroll
             for (int j = 0; j < P; ++j) d[j] = __fmaf_rn(SHORT ? ps[j] : a.pw[P - 1 - j], z, d[j]);
         }
-        if constexpr (!SHORT) {
+        if constexpr (SHORT) {
+            // explicit rows have their own values, whatever the others hold
+#pragma unroll
+            for (int r = 0; r < NEXP; ++r) {
+                if (lo) d[r] = gl[r];
+#pragma unroll
+                for (int j = 0; j < P; ++j)
+                    if (hi && j == hj - r) d[j] = gh[r];
+            }
+        } else {
             if (anylo) {
                 const float x0 = __shfl_sync(ALL, d[NEXP], max(lane - ch, 0));
                 const float y = near_lo ? __fmul_rn(kf, x0) : 0.0f;
