@@ -159,7 +159,16 @@ __global__ void initial_state_kernel(const BoxDev bx, unsigned long long seed, d
 constexpr int DIAG_THREADS = 256;
 constexpr int DIAG_REC = 10;
 
-__global__ void diag_partial_kernel(const BoxDev bx, const double *__restrict__ Q, double *partial, unsigned *seen)
+// BLOCKS: blocks per SM it is compiled for.  A row keeps nx of a block's threads
+// busy, so short rows want four blocks (64 registers); long ones run faster with
+// the 72 registers the compiler takes for three.  After eight steps, us, three
+// and four blocks: 9 x 400 x 400 675 and 492, 101 x 1001 x 51 328 and 279,
+// 128 x 256 x 256 416 and 342, 160 431 and 408, 192 480 and 479, 224 508 and 551,
+// 256 553 and 623: four up to 160 points.
+constexpr int DIAG_SHORT = 160;
+template <int BLOCKS>
+__global__ void __launch_bounds__(DIAG_THREADS, BLOCKS)
+diag_partial_kernel(const BoxDev bx, const double *__restrict__ Q, double *partial, uint4 *seen)
 {
     __shared__ double sh[DIAG_REC][DIAG_THREADS];
     const long long np = bx.np;
@@ -180,15 +189,20 @@ __global__ void diag_partial_kernel(const BoxDev bx, const double *__restrict__ 
     // rounding error, could reach the current maxima (or are not numbers);
     // the maxima are those of the FP64 values of the points that could raise
     // them, so they are the same as evaluating every point in FP64.  The
-    // thresholds are those of all warps (seen, zero at launch; a warp looks at
-    // them once a row): a warp evaluates when any lane passes, so lanes each
-    // finding maxima of their own kept it evaluating nearly every point of boxes
-    // up to 256^3 (1.14 ms there; 0.98 with the maxima of each warp, 0.71 now)
+    // thresholds are those of all warps (seen, zero at launch): a warp evaluates
+    // when any lane passes, so lanes each finding maxima of their own kept it
+    // evaluating nearly every point of boxes up to 256^3 (1.49 ms there after
+    // eight steps, 0.55 now).  A warp that has points reads them once a row, with
+    // one load that is in flight with the row's own: every warp reads the same
+    // line, L2 serves 2.7 such reads a ns, and three loads a row by every warp
+    // took longer than short rows themselves (9 x 400 x 400: 1.11 ms, 0.49 now;
+    // 0.75 with thresholds of each thread)
     float v5f = 0.0f, v6f = 0.0f, v7f = 0.0f;
     bool screening = true;
     int nseen = 0, ncand = 0;
     const float gm1f = (float)gm1, igamf = (float)igam;
-    for (int rw = blockIdx.x; rw < rows; rw += gridDim.x) {
+    for (int rw = (int)(threadIdx.x & ~31u) < nx ? blockIdx.x : rows; rw < rows; rw += gridDim.x) {
+        const uint4 all = __ldcg(seen);
         const int y = rw % ny, z = rw / ny;
         const long long base = (long long)rw * nx;
         // coordinate along gravity of the row (gravity along y or z)
@@ -200,12 +214,10 @@ __global__ void diag_partial_kernel(const BoxDev bx, const double *__restrict__ 
         // disturbances far smaller than p itself
         const double Eb_r = bx.ga != 0 && bx.E_b64 ? bx.E_b64[kr] : 0.0;
         const float cf_r = narrow_f64(gm1 * Eb_r - ph_r);
-        v5f = fmaxf(v5f, __uint_as_float(__ldcg(seen)));
-        v6f = fmaxf(v6f, __uint_as_float(__ldcg(seen + 1)));
-        v7f = fmaxf(v7f, __uint_as_float(__ldcg(seen + 2)));
         for (int xw = threadIdx.x & ~31; xw < nx; xw += blockDim.x) {
             const int x = xw + (int)(threadIdx.x & 31);
-            bool cand = false;
+            bool cand = false, rise = false;
+            float n5f = 0.0f, n6f = 0.0f, n7f = 0.0f;
             if (x < nx) {
                 const long long p = base + x;
                 const double kgh = bx.ga == 0 ? x * bx.h[0] : kgh_r;
@@ -225,6 +237,9 @@ __global__ void diag_partial_kernel(const BoxDev bx, const double *__restrict__ 
                 // binary32 ulps of |E| + |kinetic| + |p_h|, with room to spare),
                 // so Mach^2 only where p is known to 1e-4 relative
                 cand = true;
+                v5f = fmaxf(v5f, __uint_as_float(all.x));
+                v6f = fmaxf(v6f, __uint_as_float(all.y));
+                v7f = fmaxf(v7f, __uint_as_float(all.z));
                 if (screening) {
                     const double Eb = bx.ga == 0 ? (bx.E_b64 ? bx.E_b64[x] : 0.0) : Eb_r;
                     const float cf = bx.ga == 0 ? narrow_f64(gm1 * Eb - ph) : cf_r;
@@ -266,22 +281,28 @@ __global__ void diag_partial_kernel(const BoxDev bx, const double *__restrict__ 
                         v[7] = fmax(v[7], num / pr);
                         v7t = v[7] * 0.999999;
                     }
+                    // thresholds a little below the maxima; none while a maximum
+                    // is too small for the binary32 estimates to resolve
+                    const float m5 = narrow_f64(v[5]), m7 = narrow_f64(v[7]);
+                    n5f = m5 > 1e-30f ? m5 * 0.99999f : 0.0f;
+                    n6f = narrow_f64(v[6]) * 0.99999f;
+                    n7f = m7 > 1e-30f ? m7 * 0.9999f : 0.0f;
+                    rise = n5f > v5f || n6f > v6f || n7f > v7f;
                 }
             }
-            if (__any_sync(0xffffffffu, cand)) {
-                // thresholds a little below the warp's maxima (not negative, so
-                // their bit patterns are ordered as the values are); none while
-                // a maximum is too small for the binary32 estimates to resolve
-                auto raise = [&](float &t, float f, unsigned *all) {
+            if (__any_sync(0xffffffffu, rise)) {
+                // those of the warp (not negative, so their bit patterns are
+                // ordered as the values are)
+                auto raise = [&](float &t, float f, unsigned *to) {
                     const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(f));
                     if (__uint_as_float(m) > t) {
                         t = __uint_as_float(m);
-                        if ((threadIdx.x & 31) == 0) atomicMax(all, m);
+                        if ((threadIdx.x & 31) == 0) atomicMax(to, m);
                     }
                 };
-                raise(v5f, v[5] > 1e-30 ? narrow_f64(v[5]) * 0.99999f : 0.0f, seen);
-                raise(v6f, narrow_f64(v[6]) * 0.99999f, seen + 1);
-                raise(v7f, v[7] > 1e-30 ? narrow_f64(v[7]) * 0.9999f : 0.0f, seen + 2);
+                raise(v5f, n5f, &seen->x);
+                raise(v6f, n6f, &seen->y);
+                raise(v7f, n7f, &seen->z);
             }
         }
     }
@@ -381,10 +402,14 @@ cudaError_t launch_diagnostics(const BoxDev &bx, const double *Q, double *partia
                                cudaStream_t st)
 {
     // the warps' common thresholds, after the partial records and the result
-    unsigned *seen = reinterpret_cast<unsigned *>(partial + (size_t)nblk * DIAG_REC + 10);
-    cudaError_t e = cudaMemsetAsync(seen, 0, 3 * sizeof(unsigned), st);
+    // (16-byte aligned: an even number of doubles from the allocation's start)
+    uint4 *seen = reinterpret_cast<uint4 *>(partial + (size_t)nblk * DIAG_REC + 10);
+    cudaError_t e = cudaMemsetAsync(seen, 0, sizeof(uint4), st);
     if (e != cudaSuccess) return e;
-    diag_partial_kernel<<<nblk, DIAG_THREADS, 0, st>>>(bx, Q, partial, seen);
+    if (bx.n[0] <= DIAG_SHORT)
+        diag_partial_kernel<4><<<nblk, DIAG_THREADS, 0, st>>>(bx, Q, partial, seen);
+    else
+        diag_partial_kernel<3><<<nblk, DIAG_THREADS, 0, st>>>(bx, Q, partial, seen);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     diag_final_kernel<<<1, DIAG_THREADS, 0, st>>>(bx, partial, nblk, out);
