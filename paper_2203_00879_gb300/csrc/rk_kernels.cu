@@ -79,7 +79,8 @@ __global__ void prep_kernel(const BoxDev bx, const double *__restrict__ Q, T *__
 
 // Mixed-form filter (Sec. 4): the FP32 deviation D_n was filtered into Fd;
 // the state takes the change Fd - D_n in FP64, so its low-order bits survive,
-// and W0 and D_n are recomputed from the new state.
+// and W0 and D_n are recomputed from the new state.  A point's fifteen loads are
+// issued before the first conversion, whose branch loads do not move across.
 __global__ void filter_update_kernel(const BoxDev bx, double *__restrict__ Q, const float *__restrict__ Fd,
                                      float *__restrict__ W, float *__restrict__ Dn)
 {
@@ -91,9 +92,12 @@ __global__ void filter_update_kernel(const BoxDev bx, double *__restrict__ Q, co
             const long long p = (long long)rw * nx + x;
             const int kg = bx.ga == 0 ? x : (bx.ga == 1 ? y : z);
             double q[5];
+            float fd[5], dn[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k] = Q[k * np + p], fd[k] = Fd[k * np + p], dn[k] = Dn[k * np + p];
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
-                q[k] = Q[k * np + p] + widen_f32(Fd[k * np + p] - Dn[k * np + p]);
+                q[k] += widen_f32(fd[k] - dn[k]);
                 Q[k * np + p] = q[k];
             }
             prep_point<float>(bx, p, kg, q[0], q[1], q[2], q[3], q[4], W, Dn);
