@@ -393,7 +393,7 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
 #pragma unroll 1
             for (int m = n; m >= next; --m) {
                 const int sb = (m & (R - 1)) * MR_G, ib = r0 + MR_G * m;
-                const bool out = ib < emax;
+                const bool out = ib < emax, wall = low && m == 0;
 #pragma unroll
                 for (int u = MR_G - 1; u >= 0; --u) {
                     float d[NF];
@@ -402,7 +402,8 @@ __device__ __forceinline__ void march_body(const Sweep32Args &a, const unsigned 
                     // an explicit row (factor 0) has its own value whatever the
                     // rows above it hold
 #pragma unroll
-                    for (int k = 0; k < NF; ++k) X[k] = cp == 0.0f ? d[k] : __fmaf_rn(-cp, X[k], d[k]);
+                    for (int k = 0; k < NF; ++k)
+                        X[k] = u < NEXP && wall ? d[k] : __fmaf_rn(-cp, X[k], d[k]);
                     if (out && ib + u < emax) emit(ib + u, X);
                 }
             }
@@ -609,13 +610,18 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
             const float2 q0 = *reinterpret_cast<const float2 *>(t + pl + 2), q3 = *reinterpret_cast<const float2 *>(t + pr);
             w[2] = q0.x, w[3] = q0.y;
             w[12] = q3.x, w[13] = q3.y;
+            if constexpr (SHORT) {
+                // the next line's points, in the stencils of rows beyond this
+                // line's end
+                if (ok && ch == a.nch - 1) w[12] = w[13] = 0.0f;
+                if constexpr (HW > 2) w[14] = ok && ch == a.nch - 1 ? 0.0f : w[14];
+            }
         }
         float d[P], gl[NEXP], gh[NEXP];
 #pragma unroll
         for (int j = 0; j < P; ++j) {
             d[j] = sweep_rhs<MODE>(a, w + 4 + j - HW, 1);
-            // rows beyond the line's end have the next line's points in their stencils
-            if constexpr (SHORT) d[j] = j < cnt ? __fmul_rn(rt[j], d[j]) : 0.0f;
+            if constexpr (SHORT) d[j] = __fmul_rn(rt[j], d[j]);
         }
         if (anylo) {
 #pragma unroll
@@ -694,16 +700,7 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
 #pragma unroll
             for (int j = 0; j < P; ++j) d[j] = __fmaf_rn(SHORT ? ps[j] : a.pw[P - 1 - j], z, d[j]);
         }
-        if constexpr (SHORT) {
-            // explicit rows have their own values, whatever the others hold
-#pragma unroll
-            for (int r = 0; r < NEXP; ++r) {
-                if (lo) d[r] = gl[r];
-#pragma unroll
-                for (int j = 0; j < P; ++j)
-                    if (hi && j == hj - r) d[j] = gh[r];
-            }
-        } else {
+        if constexpr (!SHORT) {
             if (anylo) {
                 const float x0 = __shfl_sync(ALL, d[NEXP], max(lane - ch, 0));
                 const float y = near_lo ? __fmul_rn(kf, x0) : 0.0f;
@@ -725,6 +722,14 @@ __device__ __forceinline__ void scan_body(const Sweep32Args &a, const int wid, f
         __syncwarp();  // the neighbours have read their halo points
         *reinterpret_cast<float4 *>(t + po) = make_float4(d[0], d[1], d[2], d[3]);
         *reinterpret_cast<float4 *>(t + po + 4) = make_float4(d[4], d[5], d[6], d[7]);
+        if constexpr (SHORT) {
+            // explicit rows have their own values, whatever the others hold
+#pragma unroll
+            for (int r = 0; r < NEXP; ++r) {
+                if (lo) t[po + r] = gl[r];
+                if (hi && hj >= r && hj - r < P) t[po + hj - r] = gh[r];
+            }
+        }
     }
     __syncwarp();
 
