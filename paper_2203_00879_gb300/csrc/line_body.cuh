@@ -28,7 +28,15 @@ struct LineArgs {
     const T *b1;    // FLUX: H_b,   FILTER: E_b,   VGRAD: 1/p_b (FP32) / p_b (FP64)
     const T *b2;    // VGRAD: 1/rho_b (FP32)
     T gm2;          // VGRAD: gamma M^2 (FP64)
+    T w[2][4];      // sub-domain sweep: right-hand-side weights (nohap_solve_column)
 };
+
+// the factor on a sweep's results: 1 / h, and the flux's sign
+template <typename T, int MODE>
+__host__ __device__ __forceinline__ T line_factor(const LineArgs<T> &a)
+{
+    return MODE == MODE_FILTER ? T(1) : (MODE == MODE_FLUX ? -a.scale : a.scale);
+}
 
 // One block of the sub-domain sweep: block `vblock` of the launch grid
 // (sub-domain vblock % nsub of line tile vblock / nsub), in the block's
@@ -261,9 +269,7 @@ __device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T>
                 gs = dot_col(cs, col + (size_t)(j0s - org) * LP, lens, LP);
                 if (lene > 0) ge = dot_col(ce, col + (size_t)(j0e - org) * LP, lene, LP);
             }
-            // the factor 1 / h, and the flux's sign, are part of the solve
-            const T osc = MODE == MODE_FILTER ? T(1) : (MODE == MODE_FLUX ? -a.scale : a.scale);
-            nohap_solve_column<T, MODE>(op, col, LP, org, gs, ge, tcp, tiv, KC, rec, osc);
+            nohap_solve_column<T, MODE>(op, a.w, col, LP, org, gs, ge, tcp, tiv, KC, rec, line_factor<T, MODE>(a));
         }
     }
     __syncthreads();

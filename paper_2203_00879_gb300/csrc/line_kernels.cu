@@ -47,6 +47,10 @@ cudaError_t launch_axis(const LineOpDev &op, LineArgs<T> a, int pref_lines, cuda
     if constexpr (AXIS == 0 && MODE == MODE_FLUX) {
         if (g.xline) return launch_xline_flux<T>(op, a, g.nblk, g.threads, g.smem, st);
     }
+    for (int k = 0; k < 4; ++k) {
+        a.w[0][k] = line_factor<T, MODE>(a) * (T)op.rb[k];
+        a.w[1][k] = a.w[0][k] * (T)op.invL;
+    }
     line_kernel<T, MODE, AXIS><<<(unsigned)g.nblk, g.threads, g.smem, st>>>(op, a);
     return cudaGetLastError();
 }

@@ -57,10 +57,16 @@ __device__ __forceinline__ T dot_col(const T *c, const T *f, int len, int LP)
 
 // org: the row at col[0]; gs / ge: the end values at rows s and e (ge unused
 // when e == s); tcp / tiv: the first KC Thomas factors (the rest equal their
-// limits cpL / invL).
+// limits cpL / invL); w: the right-hand-side weights times osc, and these times
+// invL.  A single field takes them from there, kernel parameters, so that they
+// need no registers: scaled in the kernel they cost it an eighth of its warps
+// (400 x 9 x 400 along y 40.8 us, 35.1 now; 24 x 300 x 200 along x, order 3, 41.3
+// and 35.1).  Sweeps of several fields scale them in the kernel: for these the
+// parameters are slower (128^3 filter 980 against 954 us).
 template <typename T, int MODE>
-__device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, int LP, int org, T gs, T ge,
-                                                   const T *tcp, const T *tiv, int KC, const int *rec, T osc)
+__device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, const T (&w)[2][4], T *col, int LP, int org,
+                                                   T gs, T ge, const T *tcp, const T *tiv, int KC, const int *rec,
+                                                   T osc)
 {
     constexpr int W = MODE == MODE_FILTER ? 3 : 2;     // right-hand-side half-width
     constexpr int NEXP = MODE == MODE_FILTER ? 3 : 2;  // explicit rows at each wall
@@ -99,7 +105,10 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
         const T al = (T)op.alpha;
         const T gL = lo == s + 1 ? gs : exL[NEXP - 1];
         const T gR = hi == e - 1 ? ge : exH[NEXP - 1];
-        T r0 = osc * (T)op.rb[0], r1 = osc * (T)op.rb[1], r2 = osc * (T)op.rb[2], r3 = osc * (T)op.rb[3];
+        constexpr bool SINGLE = MODE == MODE_FIELD || MODE == MODE_FIELD2;
+        T b[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) b[k] = SINGLE ? w[0][k] : osc * (T)op.rb[k];
         const T cL = (T)op.cpL, iL = (T)op.invL;
         T win[2 * W + 1];
         const T *pin = col + (size_t)(lo - W - tlo) * LP;
@@ -110,22 +119,22 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
         T dprev = 0;
         // one forward row: right-hand side from the window, minus the
         // coupling `adj` to a known end value, then the elimination
-        auto right = [&] {
+        auto right = [&](const T(&b)[4]) {
             win[2 * W] = *pin;
             pin += LP;
             T rhs;
             if constexpr (MODE == MODE_FILTER)
-                rhs = r0 * win[3] + r1 * (win[4] + win[2]) + r2 * (win[5] + win[1]) + r3 * (win[6] + win[0]);
+                rhs = b[0] * win[3] + b[1] * (win[4] + win[2]) + b[2] * (win[5] + win[1]) + b[3] * (win[6] + win[0]);
             else if constexpr (MODE == MODE_FIELD2)
-                rhs = r0 * win[2] + r1 * (win[3] + win[1]) + r2 * (win[4] + win[0]);
+                rhs = b[0] * win[2] + b[1] * (win[3] + win[1]) + b[2] * (win[4] + win[0]);
             else
-                rhs = r0 * (win[3] - win[1]) + r1 * (win[4] - win[0]);
+                rhs = b[0] * (win[3] - win[1]) + b[1] * (win[4] - win[0]);
 #pragma unroll
             for (int j = 0; j < 2 * W; ++j) win[j] = win[j + 1];
             return rhs;
         };
         auto fwd = [&](T iv, T adj) {
-            const T dp = (right() - adj - al * dprev) * iv;
+            const T dp = (right(b) - adj - al * dprev) * iv;
             *pout = dp;
             pout += LP;
             dprev = dp;
@@ -137,18 +146,15 @@ __device__ __forceinline__ void nohap_solve_column(const LineOpDev &op, T *col, 
 #pragma unroll 4
         for (; r < kmid; ++r) fwd(tiv[r], T(0));
         if (r < m - 1) {
-            const T q0 = r0, q1 = r1, q2 = r2, q3 = r3;
-            r0 *= iL;
-            r1 *= iL;
-            r2 *= iL;
-            r3 *= iL;
+            T c[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) c[k] = SINGLE ? w[1][k] : b[k] * iL;
 #pragma unroll 4
             for (; r < m - 1; ++r) {
-                dprev = right() - cL * dprev;
+                dprev = right(c) - cL * dprev;
                 *pout = dprev;
                 pout += LP;
             }
-            r0 = q0, r1 = q1, r2 = q2, r3 = q3;
         }
         if (m > 1) fwd(m - 1 < KC ? tiv[m - 1] : iL, al * gR);
         // back substitution from row hi - 1 down to lo
