@@ -93,7 +93,13 @@ typedef struct {
                            /* is the mid-plane normal to it                          */
     int sub_n[3];          /* NOHAP sub-domain length per axis (>= 3); 0 or >= n:   */
                            /* one sub-domain; -1: the autotuner picks 32, 64 or 128 */
-                           /* by timing this GPU at nopcs_init                      */
+                           /* by timing this GPU at nopcs_init.  Results do not     */
+                           /* depend on it beyond rounding.  Under NOPCS_MIXED it   */
+                           /* cuts the lines of nopcs_derivative alone (FP64; FP32  */
+                           /* in the Thomas form along y and z and in the tensor-   */
+                           /* core forms): the steps' sweeps take no notice of it,  */
+                           /* and -1 is 64 (32 where n <= 64) where the FP32        */
+                           /* derivative's time does not depend on it either        */
     double Re, M, Pr, gamma;
     double suth_S;         /* Sutherland constant / T_s                             */
     double mub_scale;      /* factor on the bulk-viscosity law, Eq. reg             */

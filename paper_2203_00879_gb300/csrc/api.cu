@@ -298,10 +298,12 @@ cudaError_t refresh_mixed(BoxRes &b, cudaStream_t st)
 // ---- autotuner ---------------------------------------------------------------
 // Per axis: in the FP64 form, the flux sweep's tile width (16 or 32 lines per
 // block); where the descriptor asks with sub_n = -1, the sub-domain length
-// (32, 64 or 128), by timing the flux sweep (FP64 form, together with the tile
-// width) or the FP32 derivative (mixed form, whose flux sweeps do not depend
-// on the partition).  Under NOPCS_FORM_AUTO each axis's FP32 derivative takes
-// the Thomas, the banded or a tensor-core form, whichever measured faster.
+// (32, 64 or 128).  FP64 form: by timing the flux sweep, together with the tile
+// width.  Mixed form, whose flux sweeps do not depend on the partition: by timing
+// the FP32 derivative in the forms the context may give the axis, as far as they
+// depend on it (tune_sub_mixed).  Under NOPCS_FORM_AUTO each axis's FP32
+// derivative takes the Thomas, the banded or a tensor-core form, whichever
+// measured faster.
 // Times come from CUDA events on the context stream (one warm-up, three timed
 // launches); choices are cached per box shape for the process.  Boxes below
 // 2^20 points keep the defaults unless a sub-domain length is requested.
@@ -326,6 +328,65 @@ float time_launches(cudaStream_t st, const std::function<cudaError_t()> &fn, cud
     return ms;
 }
 
+// The FP32 derivative of axis a, launched in one of its forms: 0 Thomas, 1 3xTF32,
+// 2 banded, 3 BF16x3.
+cudaError_t launch_form(nopcs_ctx *ctx, BoxRes &b, int a, int form, const float *fin, float *fout)
+{
+    const int *n = b.dev.n;
+    switch (form) {
+    case 0: return launch_line_field<float>(b.dop32[a].dev, a, n, fin, fout, 1.0, ctx->stream);
+    case 2: return launch_band_field(b.bop[a], a, n, fin, fout, 1.0, ctx->stream);
+    default: return launch_gemm_field(b.gop[a].dev, form == 3, a, n, fin, fout, 1.0, ctx->dev_err, ctx->stream);
+    }
+}
+
+// Sub-domain length of axis a of a mixed-form box that asks for -1.  64 where n
+// allows it, unless another length makes the axis's FP32 derivative more than 3%
+// faster (more than the times of one launch differ).  The Thomas form along x
+// and the banded form take no notice of the partition: where the context's form
+// is one of them, or under NOPCS_FORM_AUTO one of them is the fastest, every
+// length would time the same launch, so 64 stays.
+nopcs_status tune_sub_mixed(nopcs_ctx *ctx, BoxRes &b, int a, const float *fin, float *fout, int &best)
+{
+    const int n = b.dev.n[a];
+    best = n > 64 ? 64 : 32;
+    if (n <= 64) return NOPCS_OK;
+    const nopcs_form f = ctx->form;
+    const bool all = f == NOPCS_FORM_AUTO;
+    auto fastest = [&](const bool (&take)[4], float &ms) {
+        ms = 1e30f;
+        for (int k = 0; k < 4; ++k) {
+            if (!take[k] || ((k & 1) && !b.gop[a].mem) || (k == 2 && !b.bop[a].mem)) continue;
+            cudaError_t e;
+            const float t = time_launches(ctx->stream, [&] { return launch_form(ctx, b, a, k, fin, fout); }, e);
+            if (e != cudaSuccess) return e;
+            if (t < ms) ms = t;
+        }
+        return cudaSuccess;
+    };
+    const bool split[4] = {a != 0 && (all || f == NOPCS_FORM_THOMAS), all || f == NOPCS_FORM_GEMM_3XTF32, false,
+                           all || f == NOPCS_FORM_GEMM_BF16X3};
+    const bool whole[4] = {all && a == 0, false, all, false};
+    if (!split[0] && !split[1] && !split[3]) return NOPCS_OK;
+    float tbest = 1e30f, tsplit = 1e30f, twhole = 1e30f;
+    for (int cand : {64, 32, 128}) {
+        if (cand >= n) continue;
+        b.sub_n[a] = cand;
+        const nopcs_status s = build_axis_ops(ctx, b, a);
+        if (s != NOPCS_OK) return s;
+        float ms;
+        CK(fastest(split, ms), "autotune");
+        if (cand == 64) CK(fastest(whole, twhole), "autotune");
+        if (ms < tsplit) tsplit = ms;
+        if (cand == 64 || ms < 0.97f * tbest) {
+            tbest = ms;
+            best = cand;
+        }
+    }
+    if (twhole <= tsplit) best = 64;
+    return NOPCS_OK;
+}
+
 nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
 {
     cudaStream_t st = ctx->stream;
@@ -340,14 +401,21 @@ nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
     for (int a = 0; a < 3; ++a) {
         const bool tune_sub = b.d.sub_n[a] == -1;
         if (!tune_sub && (b.mixed || x.np < (1LL << 20))) continue;
-        const std::string key = std::string(key0) + ",s" + std::to_string(a) + "," + std::to_string(b.d.sub_n[a]);
+        const std::string key = std::string(key0) + ",s" + std::to_string(a) + "," + std::to_string(b.d.sub_n[a]) +
+                                (b.mixed ? ",f" + std::to_string((int)ctx->form) : "");
         int best = -1;  // sub_n * 1000 + lines per block
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
             auto it = g_tune_cache.find(key);
             if (it != g_tune_cache.end()) best = it->second;
         }
-        if (best < 0) {
+        if (best < 0 && b.mixed) {
+            const nopcs_status s2 = tune_sub_mixed(ctx, b, a, fin, fout, best);
+            if (s2 != NOPCS_OK) return s2;
+            best *= 1000;
+            std::lock_guard<std::mutex> lk(g_tune_mu);
+            g_tune_cache[key] = best;
+        } else if (best < 0) {
             float tbest = 1e30f;
             std::vector<int> cands;
             if (tune_sub)
@@ -362,10 +430,8 @@ nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
                     if (s2 != NOPCS_OK) return s2;
                 }
                 for (int ln : {16, 32}) {
-                    if (b.mixed && ln == 16) continue;
                     cudaError_t e;
-                    float ms = b.mixed ? time_launches(st, [&] { return launch_line_field<float>(b.dop32[a].dev, a, x.n, fin, fout, 1.0, st); }, e)
-                                       : time_launches(st, [&] { return launch_line_flux<double>(b.dop64[a].dev, a, x, (double *)b.W, (double *)b.R, 1, st, ln); }, e);
+                    float ms = time_launches(st, [&] { return launch_line_flux<double>(b.dop64[a].dev, a, x, (double *)b.W, (double *)b.R, 1, st, ln); }, e);
                     if (e != cudaSuccess) return cuda_fail(ctx, e, "autotune");
                     if (ms < tbest) {
                         tbest = ms;
@@ -401,10 +467,10 @@ nopcs_status autotune_box(nopcs_ctx *ctx, BoxRes &b)
                 // 0 Thomas, 1 3xTF32, 2 banded, 3 BF16x3: the fastest
                 cudaError_t e[4] = {cudaSuccess, cudaSuccess, cudaSuccess, cudaSuccess};
                 float t[4];
-                t[0] = time_launches(st, [&] { return launch_line_field<float>(b.dop32[a].dev, a, x.n, fin, fout, 1.0, st); }, e[0]);
-                t[1] = b.gop[a].mem ? time_launches(st, [&] { return launch_gemm_field(b.gop[a].dev, false, a, x.n, fin, fout, 1.0, ctx->dev_err, st); }, e[1]) : 1e30f;
-                t[2] = b.bop[a].mem ? time_launches(st, [&] { return launch_band_field(b.bop[a], a, x.n, fin, fout, 1.0, st); }, e[2]) : 1e30f;
-                t[3] = b.gop[a].mem ? time_launches(st, [&] { return launch_gemm_field(b.gop[a].dev, true, a, x.n, fin, fout, 1.0, ctx->dev_err, st); }, e[3]) : 1e30f;
+                for (int k = 0; k < 4; ++k) {
+                    const bool have = k == 0 || (k == 2 ? b.bop[a].mem != nullptr : b.gop[a].mem != nullptr);
+                    t[k] = have ? time_launches(st, [&] { return launch_form(ctx, b, a, k, fin, fout); }, e[k]) : 1e30f;
+                }
                 for (cudaError_t ei : e)
                     if (ei != cudaSuccess) return cuda_fail(ctx, ei, "autotune");
                 choice = 0;
