@@ -45,6 +45,8 @@ ALG_BYTES_MIXED = {
     # instead of the five primitives the viscous stencils need
     "source_rk_update": (88 + 108 + 108 + 164) / 4.0,
 }
+# kernel launches behind one profiled launch of a kind in the mixed form (1 where not named)
+LAUNCHES_PER_KIND = {"wall_bc": 1, "filter": 4, "diagnostics": 2}
 ALG_BYTES_FP64 = {
     "prep": 40 + 48, "sweep_x": 48 + 40, "sweep_y": 48 + 80, "sweep_z": 48 + 80,
     "visc_rk_update": (188 + 228 * 2 + 148) / 4.0, "filter": 3 * 80,
@@ -485,11 +487,10 @@ def main():
     ms_prof = e0.elapsed_time(e1)
     prof = N.nopcs_profile_read(ctx, reset=True)
     N.nopcs_set_profiling(ctx, False)
-    launches_per_kind = {"prep": 1, "sweep_x": 1, "sweep_y": 1, "sweep_z": 1, "visc_rk_update": 1,
-                         "wall_bc": 3, "filter": 4, "diagnostics": 2}
-    step_launches = sum(v[1] * launches_per_kind.get(k, 1) for k, v in prof.items()
+    step_launches = sum(v[1] * LAUNCHES_PER_KIND.get(k, 1) for k, v in prof.items()
                         if k not in ("filter", "diagnostics")) / KP
-    gpu_launches = int(round(step_launches * K)) + 4 * filters_in_window + 2
+    gpu_launches = (int(round(step_launches * K)) + LAUNCHES_PER_KIND["filter"] * filters_in_window +
+                    LAUNCHES_PER_KIND["diagnostics"])
 
     # dominant kernel against the HBM roofline
     hbm, peak_kind = peaks()

@@ -1,11 +1,14 @@
-"""The source lists that tag profiler counters name every file in which a
-device function that the kind runs is defined (CPU)."""
+"""What the benchmark says of the kernels, against the sources (CPU): the lists
+that tag profiler counters name every file in which a device function that the
+kind runs is defined, and a kind counts as many launches as its launcher makes."""
 import os
 import re
 
 import pytest
 
 from paper_2203_00879_gb300 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 USES = {
     "prep": ["prep_kernel", "prep_point", "narrow_f64"],
@@ -34,3 +37,21 @@ def test_lists_name_every_source(kind):
         assert files, name
         missing = set(files) - set(build.KERNEL_FILES[kind])
         assert not missing, (kind, name, missing)
+
+
+def _launches(source, function):
+    """Kernel launches that one call of a launcher makes: the branches of an if
+    each hold one."""
+    text = open(os.path.join(build.CSRC, source)).read()
+    body = re.search(r"\n(?:template [^\n]*\n)?cudaError_t %s\(.*?\n}\n" % function, text, re.S).group(0)
+    return body.count("<<<") - len(re.findall(r"\n    else\n", body))
+
+
+def test_launches_per_kind():
+    src = open(os.path.join(ROOT, "bench.py")).read()
+    per_kind = dict(re.findall(r'"(\w+)": (\d+)', re.search(r"LAUNCHES_PER_KIND = \{(.*?)\}", src, re.S).group(1)))
+    assert int(per_kind["wall_bc"]) == _launches("rk_kernels.cu", "launch_wall_bc")
+    assert int(per_kind["diagnostics"]) == _launches("rk_kernels.cu", "launch_diagnostics")
+    # three sweeps and the update
+    assert int(per_kind["filter"]) == 3 + _launches("rk_kernels.cu", "launch_filter_update")
+    assert _launches("rk_kernels.cu", "launch_prep") == 1
