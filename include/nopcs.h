@@ -225,7 +225,9 @@ nopcs_status nopcs_set_step(nopcs_ctx *ctx, int box, long long step);
  * C rows truncated at |C| < 1e-8 (24 taps each side).  f and df are device
  * pointers of np elements, must not overlap; the work is enqueued on `stream`
  * and the call does not wait.  order 2 uses library-owned scratch of np
- * elements.  Errors: EINVAL, ECUDA.
+ * elements.  Lines are independent: an infinity or NaN in f changes the results
+ * of its own line only (which of them, beyond the stencil, depends on the form
+ * and the partition).  Errors: EINVAL, ECUDA.
  */
 enum { NOPCS_ORDER_D2_COMPACT = 3 };
 nopcs_status nopcs_derivative(nopcs_ctx *ctx, int box, int axis, int order, int dtype,
@@ -274,7 +276,10 @@ nopcs_status nopcs_rk_step(nopcs_ctx *ctx, int nsteps);
  *   NOPCS_LAUNCH_PERSISTENT: one persistent kernel per step that runs every
  *     box's phases (flux sweeps, viscous/source/RK stage, walls) from a device
  *     work list, each phase of a box after the box's previous phase, every
- *     wait bounded by wait_limit_s; results are identical to the graph's;
+ *     wait bounded by wait_limit_s; results are identical to the graph's.  It
+ *     takes about twice the graph's time on GB300 (64 uneven boxes 35.7 against
+ *     18.8 ms a step): for callers that want a step to be one launch, and a
+ *     bounded wait reported by nopcs_synchronize, rather than the fastest one;
  *   NOPCS_LAUNCH_PERSISTENT_WITHHOLD: as PERSISTENT, but box 0's first
  *     dependency is never satisfied -- for testing the bounded wait: the
  *     kernel gives up after wait_limit_s and returns, nopcs_synchronize

@@ -14,6 +14,14 @@
 // start from the explicit closure rows with the tabulated factors and are
 // those of the Thomas algorithm.
 //
+// Lines are independent, also where they hold infinities or NaN: whatever a
+// kernel takes from a neighbouring thread or lane of another line is left out by
+// selection, never by a factor of zero.  Within its line such a value reaches
+// as far as the recurrence carries it: in a march the rest of its segment (a
+// whole line where lines are not cut) and the 24 rows around, along x the three
+// chunks of 8 on either side; explicit rows next to a wall only through their
+// closure.
+//
 // Two kernels use this:
 //   march_body (lines along y, z): a thread walks one line; consecutive
 //     threads take consecutive lines, so loads and stores coalesce, and no
@@ -143,7 +151,6 @@ __device__ __forceinline__ float sweep_rhs(const Sweep32Args &a, const float *w,
     }
 }
 
-constexpr int MARCH_TPB = 64;  // lines per block of a stand-alone march
 constexpr int SCAN_WARPS = 4;  // warps per block of a stand-alone scan
 
 // Host: the operator's coefficients with `scale` folded in (false if its
