@@ -50,11 +50,11 @@ struct LedgerScope {
 // Device registers of a box.
 //   FP64 form: Q = Qn, Qs, acc (15 FP64 fields); W (6 FP64); R (5 FP64).
 //   Mixed form: Q = Qn (5 FP64 fields); W = slab of two FP32 primitive sets
-//     W0, W1 of five fields each in six slots (12 in all, so that the bytes a
-//     point that memory limits are planned with stay as they are); R = slab of
-//     R, K, Dn (15 FP32 fields).  Between
-//     steps W0 and Dn hold the primitives and the base deviation of Qn, and
-//     the filter borrows both slabs as FP64 temporaries.
+//     W0, W1 of five fields each, allocated as twelve (no kernel needs the
+//     other two: a job's memory limit admits what it always has and no more,
+//     148 bytes a point); R = slab of R, K, Dn (15 FP32 fields).  Between steps
+//     W0 and Dn hold the primitives and the base deviation of Qn; the filter
+//     borrows W0, R and K for its FP32 fields.
 //   Compact viscous terms (visc_compact): Gv, 12 fields of the stage's
 //     precision holding the gradients of u, v, w, T, then the viscous fluxes.
 struct BoxRes {

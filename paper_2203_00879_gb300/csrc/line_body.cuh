@@ -340,12 +340,12 @@ __device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T>
 
 // ---- whole-line sweep along x -------------------------------------------------
 // Along x a grid line is contiguous in memory and short enough (N x 5 fields
-// x 4 B = 20 KB at N = 1024) for a block to stage LINES whole lines at once.
-// Every point is then loaded once -- a sub-domain tile also stages the 2 x 24
-// end-row support points of its neighbours, 1.75 times its own points at
+// x 8 B = 40 KB at N = 1024) for a block to stage a whole line at once.
+// Every point is then loaded once -- a sub-domain tile also reads the 2 x 48
+// end-row support points of its neighbours, 2.5 times its own points at
 // sub-domains of 64 -- and the end rows read their supports from the staged
-// lines instead of summing partial products across a warp.  Each thread
-// solves one (line, field, sub-domain) column in three phases separated by
+// line instead of summing partial products across a warp.  Each thread
+// solves one (field, sub-domain) column in three phases separated by
 // barriers, so that no column reads a row another column has overwritten:
 //   A. the two end values g_i = sum_j C_ij f_j (Eq. CS:fpCf_i) and any
 //      explicit wall row, from the staged inputs;
@@ -353,9 +353,9 @@ __device__ __forceinline__ void line_body(const LineOpDev &op, const LineArgs<T>
 //      e+1, and the only rows of other columns among them (s-1 and e+1) are
 //      their end rows, which phase B never writes;
 //   C. the end and wall values into their rows.
-// The layout is [field][line][row] with one pad word per 32 rows and a line
+// The layout is [field][row] with one pad word per 32 rows and a field
 // pitch chosen on the host (LineOpDev::xpitch) so that the columns a warp's
-// threads take (neighbouring sub-domains, then the next line) fall in
+// threads take (neighbouring sub-domains, then the next field) fall in
 // different banks.  The line's end-row taps (a few KB) are copied to shared
 // memory once per block: the threads of a warp read the taps of different
 // sub-domains, which from global memory would touch a cache line each.
@@ -381,28 +381,25 @@ __device__ __forceinline__ void xline_flux_point(const LineArgs<T> &a, T *d, con
 
 template <typename T>
 __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const LineArgs<T> &a, T *sm,
-                                                  const T *ctab, const T *tcp, const T *tiv, const int line0,
-                                                  const int nl);
+                                                  const T *ctab, const T *tcp, const T *tiv, const int base);
 
-// One block of the whole-line x sweep: lines vblock * LINES .. + LINES - 1,
-// in the block's dynamic shared memory.
+// One block of the whole-line x sweep: one line (= y + ny z), in the block's
+// dynamic shared memory.
 template <typename T>
-__device__ __forceinline__ void xline_body(const LineOpDev &op, const LineArgs<T> &a, const int vblock)
+__device__ __forceinline__ void xline_body(const LineOpDev &op, const LineArgs<T> &a, const int line)
 {
     extern __shared__ __align__(32) unsigned char smraw[];
     constexpr int NF = 5, NIN = 6;
     constexpr int U = 4;     // staged points in flight per thread and field
     const int N = op.N;      // = nx
-    const int nx = a.n[0], ny = a.n[1];
-    const int LINES = a.lines, LS = a.rt;  // lines per block, line pitch (padded)
-    const size_t FS = (size_t)LINES * LS;
+    const int ny = a.n[1];
+    const size_t FS = a.rt;  // field pitch (padded)
     const int KC = sizeof(T) == 8 ? op.kconv64 : op.kconv32;
     T *sm = reinterpret_cast<T *>(smraw);
     T *ctab = sm + NF * FS;  // end-row taps
     T *tcp = ctab + op.ncoef;
     T *tiv = tcp + KC;
-    const int line0 = vblock * LINES;
-    const int nl = min(LINES, ny * a.n[2] - line0);
+    const int base = line * N;
     {
         const T *cpp = cp_ptr<T>(op), *ivp = inv_ptr<T>(op), *cf = coef_ptr<T>(op);
         for (int k = threadIdx.x; k < KC; k += blockDim.x) {
@@ -411,56 +408,48 @@ __device__ __forceinline__ void xline_body(const LineOpDev &op, const LineArgs<T
         }
         for (int k = threadIdx.x; k < op.ncoef; k += blockDim.x) ctab[k] = cf[k];
     }
-    // ---- stage the lines: consecutive threads take consecutive points ----
-    for (int l = 0; l < nl; ++l) {
-        const int line = line0 + l;  // = y + ny z
-        const int gl = a.ga == 1 ? line % ny : line / ny;  // coordinate along gravity (y or z)
-        const int base = line * nx;
-        for (int g0 = threadIdx.x; g0 < N; g0 += U * blockDim.x) {
-            T v[U][NIN];
+    // ---- stage the line: consecutive threads take consecutive points ----
+    const int gl = a.ga == 1 ? line % ny : line / ny;  // coordinate along gravity (y or z)
+    for (int g0 = threadIdx.x; g0 < N; g0 += U * blockDim.x) {
+        T v[U][NIN];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int g = g0 + u * (int)blockDim.x;
-                if (g < N) {
+        for (int u = 0; u < U; ++u) {
+            const int g = g0 + u * (int)blockDim.x;
+            if (g < N) {
 #pragma unroll
-                    for (int k = 0; k < NIN; ++k) v[u][k] = a.in[k][base + g];
-                }
+                for (int k = 0; k < NIN; ++k) v[u][k] = a.in[k][base + g];
             }
+        }
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int g = g0 + u * (int)blockDim.x;
-                if (g >= N) continue;
-                T *d = sm + (size_t)l * LS + xrow(g);
-                xline_flux_point(a, d, FS, v[u], a.ga == 0 ? g : gl);
-            }
+        for (int u = 0; u < U; ++u) {
+            const int g = g0 + u * (int)blockDim.x;
+            if (g >= N) continue;
+            xline_flux_point(a, sm + xrow(g), FS, v[u], a.ga == 0 ? g : gl);
         }
     }
     __syncthreads();
-    xline_solve_store<T>(op, a, sm, ctab, tcp, tiv, line0, nl);
+    xline_solve_store<T>(op, a, sm, ctab, tcp, tiv, base);
 }
 
-// The solve and the store of the whole-line x sweep, once lines line0 ..
-// line0 + nl - 1 are staged in the tile sm (and a barrier has passed): the
-// columns, thread c solving sub-domain c % nsub of line (c / nsub) % nl, field
-// c / (nsub nl), in phases A-C, then the rows scaled by 1/h into the outputs.
+// The solve and the store of the whole-line x sweep, once the line is staged in
+// sm (and a barrier has passed): the columns, thread c solving sub-domain
+// c % nsub of field c / nsub, in phases A-C, then the rows scaled by 1/h into the
+// outputs, from element base on.
 template <typename T>
 __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const LineArgs<T> &a, T *sm,
-                                                  const T *ctab, const T *tcp, const T *tiv, const int line0,
-                                                  const int nl)
+                                                  const T *ctab, const T *tcp, const T *tiv, const int base)
 {
     constexpr int NF = 5;
     constexpr int NEXP = 2;  // explicit rows at each wall (derivative)
     const int N = op.N;      // = nx
-    const int nx = a.n[0];
-    const int LINES = a.lines, LS = a.rt;
-    const size_t FS = (size_t)LINES * LS;
+    const size_t FS = a.rt;
     const int KC = sizeof(T) == 8 ? op.kconv64 : op.kconv32;
     const int nsub = op.nsub;
     const int c = threadIdx.x;
-    const bool active = c < nsub * NF * nl;
-    const int b = c % nsub, l = (c / nsub) % max(nl, 1), f = c / (nsub * max(nl, 1));
+    const bool active = c < nsub * NF;
+    const int b = c % nsub, f = c / nsub;
     const int *rec = op.sub + b * SUB_REC;
-    T *col = sm + (size_t)f * FS + (size_t)l * LS;
+    T *col = sm + (size_t)f * FS;
     const int s = rec[0], e = rec[1], lo = rec[10], hi = rec[11];
     T gs = 0, ge = 0;
     T exL[NEXP], exH[NEXP];
@@ -565,20 +554,16 @@ __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const Lin
     }
     __syncthreads();
     // ---- store (scaled by 1/h; the flux sweep stores -dF/dx into R) ----
-    for (int ll = 0; ll < nl; ++ll) {
-        const int base = (line0 + ll) * nx;
-        const T *src = sm + (size_t)ll * LS;
-        for (int g = threadIdx.x; g < N; g += blockDim.x) {
-            const int o = base + g;
-            const int q = xrow(g);
+    for (int g = threadIdx.x; g < N; g += blockDim.x) {
+        const int o = base + g;
+        const int q = xrow(g);
 #pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                const T v = -src[(size_t)k * FS + q] * a.scale;
-                if (a.first)
-                    a.out[k][o] = v;
-                else
-                    atomicAdd(&a.out[k][o], v);
-            }
+        for (int k = 0; k < 5; ++k) {
+            const T v = -sm[(size_t)k * FS + q] * a.scale;
+            if (a.first)
+                a.out[k][o] = v;
+            else
+                atomicAdd(&a.out[k][o], v);
         }
     }
 }
@@ -586,10 +571,7 @@ __device__ __forceinline__ void xline_solve_store(const LineOpDev &op, const Lin
 
 // ---- launch geometry (host) ----------------------------------------------------
 constexpr size_t SMEM_BUDGET = 200 * 1024;
-// whole-line x flux sweep: at most this much shared memory per block, and
-// several lines per block only while a block stays below the second figure
-constexpr size_t XLINE_SMEM = 100 * 1024, XLINE_SMEM_MULTI = 48 * 1024;
-constexpr int XLINE_MAX_LINES = 1;  // up to 4 (LineOpDev::xpitch)
+constexpr size_t XLINE_SMEM = 100 * 1024;  // whole-line x flux sweep: most shared memory of a block
 
 inline int pick_lines(int pref, int rw, int nf, size_t esz)
 {
@@ -630,20 +612,14 @@ bool line_grid(const LineOpDev &op, LineArgs<T> &a, int pref_lines, LineGrid &g)
     const bool filled = op.N < 48 * op.nsub ? 5 * columns >= 4 * lanes
                                             : op.N < 96 * op.nsub && 10 * columns >= 9 * lanes;
     if (AXIS == 0 && MODE == MODE_FLUX && columns >= 50 && filled) {
-        for (int L = XLINE_MAX_LINES; L >= 1; --L) {
-            const int pitch = op.xpitch[L - 1];
-            const size_t bytes = ((size_t)NF * L * pitch + (size_t)op.ncoef + 2 * (size_t)kc) * sizeof(T);
-            const int cols = op.nsub * NF * L;
-            if (bytes > XLINE_SMEM || cols > 1024) continue;
-            if (L > 1 && bytes > XLINE_SMEM_MULTI) continue;
-            a.lines = L;
-            a.rt = pitch;
-            int threads = (cols + 31) / 32 * 32;
-            if (threads < 128) threads = 128;
-            g.threads = threads;
+        const size_t bytes = ((size_t)NF * op.xpitch + (size_t)op.ncoef + 2 * (size_t)kc) * sizeof(T);
+        if (bytes <= XLINE_SMEM && columns <= 1024) {
+            a.lines = 1;
+            a.rt = op.xpitch;
+            g.threads = lanes < 128 ? 128 : lanes;
             g.smem = bytes;
             g.xline = true;
-            g.nblk = ((long long)a.n[1] * a.n[2] + L - 1) / L;
+            g.nblk = (long long)a.n[1] * a.n[2];
             return g.nblk <= 0x7fffffffLL;
         }
     }

@@ -85,7 +85,7 @@ struct LineOpDev {
     int N, nsub, nexp, maxm, max_tile, max_taps, max_win;
     int kconv64, kconv32;
     int ncoef;          // end-row taps in the coef tables
-    int xpitch[4];      // whole-line x flux sweep: line pitch for 1..4 lines per block
+    int xpitch;         // whole-line x flux sweep: pitch of a field's line
     double cpL, invL;  // limits of the Thomas factors
     double alpha;
     double rb[4];
