@@ -32,7 +32,7 @@
 //     alternating load, solve and store phases.
 //   scan_body (lines along x): a lane solves 8 consecutive points and takes
 //     the recurrences' state from its three neighbour lanes by shuffles.
-//     1.99 ms (40 B a point, 0.79 of the copy bandwidth; two thirds of the
+//     2.00 ms (40 B a point, 0.79 of the copy bandwidth; two thirds of the
 //     issue slots and three quarters of the shared-memory cycles used) against
 //     3.71 for whole lines in block-wide phases.
 // One field at 512^3 (8 B a point), x, y, z: 239, 240, 243 us against 469, 546,
