@@ -29,10 +29,34 @@ __device__ __forceinline__ void coords(const BoxDev &bx, long long p, int c[3])
 // rho - rho_b and E - E_b in FP64 and the rest in FP32, using
 // p - p_b = (gamma - 1)(E - E_b - rho |V|^2 / 2); it keeps the first five.
 // ---------------------------------------------------------------------------
-// W (and the deviation D_n, mixed form) of one point of the FP64 state
-template <typename T>
-__device__ __forceinline__ void prep_point(const BoxDev &bx, long long p, int kg, double r, double mx, double my,
-                                           double mz, double E, T *__restrict__ W, float *__restrict__ Dn)
+// The base state at gravity coordinate kg (mixed form), read where it is used, or
+// ahead, with a point's other loads: the integer conversions branch, and no load
+// moves across a branch (filter of 64 x 64 x 2048: 830 us with the base read where it
+// is used, 622 ahead; of no use to rows that fill their blocks).
+struct BaseAt {
+    const BoxDev &bx;
+    int kg;
+    __device__ __forceinline__ double rho() const { return bx.rho_b64[kg]; }
+    __device__ __forceinline__ double E() const { return bx.E_b64[kg]; }
+    __device__ __forceinline__ float rho32() const { return bx.rho_b32[kg]; }
+};
+struct BaseAhead {
+    double r, e;
+    float r32;
+    __device__ __forceinline__ BaseAhead(const BoxDev &bx, int kg)
+        : r(bx.rho_b64[kg]), e(bx.E_b64[kg]), r32(bx.rho_b32[kg])
+    {
+    }
+    __device__ __forceinline__ double rho() const { return r; }
+    __device__ __forceinline__ double E() const { return e; }
+    __device__ __forceinline__ float rho32() const { return r32; }
+};
+
+// W (and the deviation D_n, mixed form) of one point of the FP64 state.  CVT:
+// hardware conversions to binary32 (the same results).
+template <typename T, bool CVT, class Base>
+__device__ __forceinline__ void prep_point(const BoxDev &bx, long long p, int kg, const Base &b, double r, double mx,
+                                           double my, double mz, double E, T *__restrict__ W, float *__restrict__ Dn)
 {
     const long long np = bx.np;
     if constexpr (sizeof(T) == 8) {
@@ -47,10 +71,10 @@ __device__ __forceinline__ void prep_point(const BoxDev &bx, long long p, int kg
     } else {
         // deviation of the state from the hydrostatic base (mixed form), then
         // the primitives from it exactly as the stage kernels form them
-        const float D[5] = {narrow_f64(r - bx.rho_b64[kg]), narrow_f64(mx), narrow_f64(my), narrow_f64(mz),
-                            narrow_f64(E - bx.E_b64[kg])};
+        auto f32 = [](double d) { return CVT ? (float)d : narrow_f64(d); };
+        const float D[5] = {f32(r - b.rho()), f32(mx), f32(my), f32(mz), f32(E - b.E())};
         float Wv[5];
-        prim_from_deviation(bx.rho_b32[kg], (float)(bx.gamma - 1.0), D, Wv);
+        prim_from_deviation(b.rho32(), (float)(bx.gamma - 1.0), D, Wv);
 #pragma unroll
         for (int k = 0; k < 5; ++k) W[k * np + p] = Wv[k];
         if (Dn) {
@@ -60,8 +84,14 @@ __device__ __forceinline__ void prep_point(const BoxDev &bx, long long p, int kg
     }
 }
 
-// grid-stride over (y, z) rows, threads along x: no 64-bit division per point
-template <typename T>
+// grid-stride over (y, z) rows, threads along x: no 64-bit division per point.
+// Mixed form: hardware conversions (CVT) for rows of up to 64 points, which leave
+// most of a block's threads idle, and for fewer rows than SMs: there the latency of
+// a row counts and not the FP64 pipe.  set_state, us, hardware and integer
+// conversions: 9 x 400 x 400 165 and 192, 64 x 256 x 256 141 and 150, 96 189 and 187, 128
+// 236 and 226, 192 331 and 320, 321 x 257 x 203 550 and 525; 4000 x 5 x 5 30 and 35.
+constexpr int PREP_SHORT = 64, PREP_ROWS = 152;
+template <typename T, bool CVT>
 __global__ void prep_kernel(const BoxDev bx, const double *__restrict__ Q, T *__restrict__ W,
                             float *__restrict__ Dn)
 {
@@ -72,7 +102,7 @@ __global__ void prep_kernel(const BoxDev bx, const double *__restrict__ Q, T *__
         for (int x = threadIdx.x; x < nx; x += blockDim.x) {
             const long long p = (long long)rw * nx + x;
             const int kg = bx.ga == 0 ? x : (bx.ga == 1 ? y : z);
-            prep_point<T>(bx, p, kg, Q[p], Q[np + p], Q[2 * np + p], Q[3 * np + p], Q[4 * np + p], W, Dn);
+            prep_point<T, CVT>(bx, p, kg, BaseAt{bx, kg}, Q[p], Q[np + p], Q[2 * np + p], Q[3 * np + p], Q[4 * np + p], W, Dn);
         }
     }
 }
@@ -91,6 +121,7 @@ __global__ void filter_update_kernel(const BoxDev bx, double *__restrict__ Q, co
         for (int x = threadIdx.x; x < nx; x += blockDim.x) {
             const long long p = (long long)rw * nx + x;
             const int kg = bx.ga == 0 ? x : (bx.ga == 1 ? y : z);
+            const BaseAhead b(bx, kg);
             double q[5];
             float fd[5], dn[5];
 #pragma unroll
@@ -100,7 +131,7 @@ __global__ void filter_update_kernel(const BoxDev bx, double *__restrict__ Q, co
                 q[k] += widen_f32(fd[k] - dn[k]);
                 Q[k * np + p] = q[k];
             }
-            prep_point<float>(bx, p, kg, q[0], q[1], q[2], q[3], q[4], W, Dn);
+            prep_point<float, false>(bx, p, kg, b, q[0], q[1], q[2], q[3], q[4], W, Dn);
         }
     }
 }
@@ -373,7 +404,10 @@ static int row_grid(const BoxDev &bx)
 template <typename T>
 cudaError_t launch_prep(const BoxDev &bx, const double *Q, T *W, float *Dn, cudaStream_t st)
 {
-    prep_kernel<T><<<row_grid(bx), 256, 0, st>>>(bx, Q, W, Dn);
+    if (sizeof(T) == 4 && (bx.n[0] <= PREP_SHORT || bx.n[1] * bx.n[2] < PREP_ROWS))
+        prep_kernel<T, sizeof(T) == 4><<<row_grid(bx), 256, 0, st>>>(bx, Q, W, Dn);
+    else
+        prep_kernel<T, false><<<row_grid(bx), 256, 0, st>>>(bx, Q, W, Dn);
     return cudaGetLastError();
 }
 
